@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -24,8 +25,10 @@ enum Stage { ST_PREDICT = 0, ST_FORCE, ST_REDUCE, ST_BATCHED, ST_VJP, ST_OTHER, 
 constexpr int kEventRing = 4096;
 constexpr int kStagesDevice = 3;       // must equal sp2::kStages of sp2_device.cuh
 constexpr int kFusedStagesDevice = 2;  // must equal sp2::kFusedStages of sp2_device.cuh
-// largest (sinks of one i-block) x (slices) reduced inside the pass kernel
+// largest (sinks of one i-block) x (slices) that a device-count pass reduces itself,
+// and that the split last wave of a pass over whole i-blocks may have
 constexpr int64_t kFusedReduceMaxValues = 16384;
+constexpr size_t kSmemPerSm = 228 * 1024;  // shared memory of an SM
 
 }  // namespace
 
@@ -85,6 +88,7 @@ struct sp2_ctx {
     std::vector<void *> owned;       // everything allocated (for close)
 
     std::map<int64_t, sp2_launch> tuned;  // key: tune_key(n_i, n_j)
+    std::map<std::array<int64_t, 5>, sp2_launch> shapes;  // default shapes of the sizes seen (shape_for)
     // profiling: per stage a ring of (start, stop) event pairs
     std::vector<cudaEvent_t> ev[ST_COUNT];
     int64_t ev_count[ST_COUNT] = {};
@@ -222,34 +226,127 @@ sp2_status check_launch(sp2_ctx *c, const sp2_launch &L) {
     return SP2_OK;
 }
 
-// Default launch shape.  Sinks first: when they do not fill one CTA, several
-// threads share a sink (j_lanes, the paper's 2D thread blocks) and the CTA
-// shrinks; then source slices (the source split) until there are ~4 work
-// items per resident CTA, so the dynamic queue balances the SMs.
-sp2_launch heuristic(const sp2_ctx *c, int kind, int mixed, int64_t n_i, int64_t n_j) {
-    sp2_launch L{};
-    L.threads = 256;
-    L.i_per_thread = (kind == K_FORCE && mixed) ? 2 : 1;
-    L.j_tile = 128;
-    L.j_lanes = 1;
-    L.ctas_per_sm = 0;
-    while (L.j_lanes < 32 && static_cast<int64_t>(L.threads / L.j_lanes) * L.i_per_thread > n_i) {
-        L.j_lanes *= 2;
-        L.i_per_thread = 1;
+// The sums of the mixed passes are rounded to FP32 per group of sources: chunks
+// of 8 sources of one lane, folded into a second level that goes into the
+// double-single totals after 64 of the lane's sources or more, at a tile end,
+// and at the end of a group of `group` sources.  Default shapes keep these
+// groups a function of the sink and source counts alone (lanes per sink, tile and
+// group below), so the results of a call do not depend on how its work is split
+// over the GPU (the FP64 passes have no such level).  Lanes share a sink when
+// there are fewer sinks than a CTA holds.
+struct Grouping {
+    int jl, tile;
+    int64_t group;  // sources, a multiple of the tile
+};
+Grouping grouping(const sp2_ctx *c, int kind, int64_t n_i, int64_t n_j) {
+    int threads = 256, ipt = kind == K_FORCE ? 2 : 1;
+    Grouping g{1, 128, 0};
+    while (g.jl < 32 && static_cast<int64_t>(threads / g.jl) * ipt > n_i) {
+        g.jl *= 2;
+        ipt = 1;
     }
-    while (L.threads > 32 && L.threads / 2 >= L.j_lanes &&
-           static_cast<int64_t>(L.threads / 2 / L.j_lanes) * L.i_per_thread >= n_i)
-        L.threads /= 2;
-    L.j_tile = std::max(L.j_tile, 8 * L.j_lanes);
-    const int64_t sinks_per_cta = static_cast<int64_t>(L.threads / L.j_lanes) * L.i_per_thread;
-    const int64_t n_iblk = ceil_div(n_i, sinks_per_cta);
-    const int64_t cta_slots = static_cast<int64_t>(c->sm_count) * std::max(1, 512 / L.threads);
-    int64_t split = ceil_div(4 * cta_slots, n_iblk);
-    const int64_t max_split = std::max<int64_t>(1, n_j / (2 * L.j_tile));
-    split = std::max<int64_t>(1, std::min(split, max_split));
-    if (n_iblk >= 4 * cta_slots) split = 1;
-    L.split_j = static_cast<int>(std::min<int64_t>(split, 65536));
-    return L;
+    while (threads > 32 && threads / 2 >= g.jl && static_cast<int64_t>(threads / 2 / g.jl) * ipt >= n_i) threads /= 2;
+    g.tile = std::max(g.tile, 8 * g.jl);
+    const int64_t n_iblk = ceil_div(n_i, static_cast<int64_t>(threads / g.jl) * ipt);
+    const int64_t slots = static_cast<int64_t>(c->sm_count) * std::max(1, 512 / threads);
+    const int64_t groups = std::max<int64_t>(1, std::min(ceil_div(4 * slots, n_iblk), n_j / (2 * g.tile)));
+    g.group = n_iblk >= 4 * slots ? ceil_div(n_j, g.tile) * g.tile : ceil_div(ceil_div(n_j, groups), g.tile) * g.tile;
+    // with 64 sources per lane and tile the totals are updated at every tile end anyway
+    if (g.tile / g.jl >= 64) g.group = g.tile;
+    return g;
+}
+
+// Dynamic shared memory of a pass launch (defined below).
+size_t pass_smem_bytes(int kind, int order, int mixed, int tile, int rb, int threads, int ipt, int fused,
+                       int fused_stages);
+
+// Default launch shape: the one with the smallest estimated time among the CTA
+// forms below (mixed: within the lanes, tile and groups of grouping()).  The
+// estimate (microseconds) is that of the SM with the most work items,
+// ceil(items / SMs): its interactions (empty sink slots and the slice rounded up
+// to whole tiles included) at the rate of a full SM, less when few warps are
+// resident or lanes share sinks; a fixed time per round of resident CTAs and per
+// tile; the prediction, in place when all sinks fit one i-block; and the
+// reduction of the slices.  The constants were fitted to 8600 measured shapes at
+// 28 sizes (512 to 131072 sources, 1 to 50000 sinks, every order and precision);
+// the shape chosen there is 3 to 4 % slower than the fastest one measured on
+// average and 17 % at most.  Against one fixed form per sink count (about four
+// items per resident CTA): 1024 sinks and sources in FP64 649 -> 95 us a step,
+// 61 sinks on 131072 sources 61 -> 49 us, 1000 on 100003 216 -> 190 us, 131072
+// on 131072 21.2 -> 20.1 ms, 4096 on 65536 at order 6 715 -> 610 us.
+struct ShapeRates {
+    double per_us;    // interactions per microsecond and SM
+    int warps[2];     // resident warps per SM of the kernels with one and two sinks per thread
+    double per_lane;  // extra work per additional lane that shares a sink (merging, conflicting reads)
+};
+constexpr ShapeRates kRatesMixed2 = {7500, {24, 16}, 0.06};
+constexpr ShapeRates kRatesMixed4 = {4700, {16, 16}, 0.05};
+constexpr ShapeRates kRatesMixed6 = {2800, {16, 8}, 0.05};
+constexpr ShapeRates kRatesVjp = {2000, {16, 8}, 0.05};
+constexpr ShapeRates kRatesFp64[4] = {{130, {24, 16}, 0.0},   // order 2
+                                      {100, {24, 16}, 0.0},   // order 4
+                                      {62, {16, 12}, 0.0},    // order 6
+                                      {40, {16, 8}, 0.0}};    // adjoint
+
+sp2_launch heuristic(const sp2_ctx *c, int kind, int order, int mixed, int64_t n_i, int64_t n_j, int nn, int nb,
+                     const Grouping &g) {
+    const ShapeRates &R = !mixed ? kRatesFp64[kind == K_VJP ? 3 : order / 2 - 1]
+                          : kind == K_VJP ? kRatesVjp
+                          : order == 6    ? kRatesMixed6
+                          : order == 2    ? kRatesMixed2
+                                          : kRatesMixed4;
+    const int rb = kind == K_VJP ? vjp_record_bytes(mixed) : record_bytes(order, mixed);
+    const int fields = (kind == K_VJP ? 7 : order == 6 ? 10 : order == 2 ? 4 : 7) + nn;
+    const bool can_fuse = mixed && kind == K_FORCE;
+    const int64_t sms = c->sm_count;
+    sp2_launch best{};
+    double best_us = 1e300;
+    for (int threads = 256; threads >= (mixed ? 128 : 64); threads /= 2)
+        for (int ipt = 1; ipt <= (can_fuse && !nb ? 2 : 1); ++ipt)
+            for (int jl = mixed ? g.jl : 1; jl <= (mixed ? g.jl : 32); jl *= 2) {
+                const int64_t spc = threads / jl * ipt, n_iblk = ceil_div(n_i, spc);
+                // (half of the sink slots empty: another form does the same with fewer idle lanes)
+                if (spc >= 2 * n_i && threads > (mixed ? 128 : 64) && (mixed || jl < 32)) continue;
+                if (!mixed && jl > 1 && n_iblk > 8 * sms) continue;
+                const int fused = can_fuse && n_iblk == 1;
+                const int warps = ipt == 1 ? R.warps[0] : fused ? 8 : order == 4 && !nn ? 12 : R.warps[1];
+                for (int tile = mixed ? g.tile : std::max(64, 8 * jl); tile <= (mixed ? g.tile : 512); tile *= 2) {
+                    const int64_t unit = mixed ? g.group : tile;
+                    const size_t smem = pass_smem_bytes(kind, order, mixed, tile, rb, threads, ipt, fused, 2);
+                    const int64_t occ = std::min<int64_t>(std::max(1, warps * 32 / threads),
+                                                          static_cast<int64_t>(kSmemPerSm / (smem + 2048)));
+                    if (occ < 1) continue;
+                    for (int per_sm : {1, 2, 3, 4, 6, 8, 12, 16, 32}) {
+                        int64_t split = std::max<int64_t>(1, per_sm * sms / n_iblk);
+                        const bool last = split > n_j / unit;
+                        split = std::min(split, ceil_div(n_j, unit));
+                        const int64_t slice = ceil_div(ceil_div(n_j, split), unit) * unit;
+                        split = ceil_div(n_j, slice);
+                        const int64_t load = ceil_div(n_iblk * split, sms), conc = std::min(load, occ);
+                        const double w = static_cast<double>(conc * threads / 32);
+                        // FP32 needs some 16 warps to fill the pipe, the 64 times slower FP64 pipe four
+                        const double eff = mixed ? std::pow(std::min(w, 16.0) / 16.0, 0.2) * std::sqrt(std::min(w, 8.0) / 8.0)
+                                                 : std::min(w, 4.0) / 4.0;
+                        double us = static_cast<double>(load * slice) *
+                                    (static_cast<double>(spc) * (1.0 + R.per_lane * (jl - 1)) + (fused ? 9.5 : 0.39 * jl)) /
+                                    (R.per_us * eff);
+                        if (ipt == 2) us *= nn ? 0.89 : 0.74;  // (each source read from shared memory serves two sinks)
+                        us += static_cast<double>(ceil_div(load, occ)) *
+                              ((fused ? 1.4 : mixed ? 3.0 : 6.0) +
+                               (fused ? 0.92 : 0.07) * static_cast<double>(slice / tile) / static_cast<double>(conc));
+                        if (!fused && can_fuse) us += 2.7;
+                        if (split > 1)
+                            us += 4.7 + 0.011 * static_cast<double>(split) +
+                                  4.6e-6 * static_cast<double>(split * fields) * static_cast<double>(n_i);
+                        if (us < best_us) {
+                            best_us = us;
+                            best = sp2_launch{threads, ipt, jl, tile, static_cast<int>(std::min<int64_t>(split, 65536)), 0};
+                        }
+                        if (last) break;  // no further slices to cut
+                    }
+                }
+            }
+    return best;
 }
 
 // Launch one persistent pass (force or VJP policy) plus its reduction.
@@ -272,13 +369,37 @@ struct PassOut {
 // prediction is fused: the pass predicts each tile in shared memory), for the mixed force passes one tile of
 // pair records, and for the mixed policies the 8-byte running totals of every
 // (thread, sink, field).
-size_t pass_smem_bytes(int kind, int order, int mixed, int tile, int rb, int threads, int ipt, int fused = 0,
-                       int fused_stages = kFusedStagesDevice) {
+size_t pass_smem_bytes(int kind, int order, int mixed, int tile, int rb, int threads, int ipt, int fused,
+                       int fused_stages) {
     const size_t ring = fused ? static_cast<size_t>(fused_stages) * tile * 16 * dscache_words(order)
                               : static_cast<size_t>(kStagesDevice) * tile * rb;
     const size_t pairs = mixed ? static_cast<size_t>(tile) * rb : 0;  // both mixed policies evaluate source pairs
     const int ns = (kind == K_VJP) ? 7 : (order == 6 ? 10 : (order == 2 ? 4 : 7));
     return ring + pairs + (mixed ? static_cast<size_t>(threads) * ipt * ns * 8 : 0);
+}
+
+// The shape of a pass: the tuned one for the bucket of its sizes, else the
+// default (a bounded table of those computed, keyed by sizes only; *group: see
+// grouping()).
+sp2_launch shape_for(sp2_ctx *c, int kind, int order, int mixed, int64_t n_i, int64_t n_j, int nn, int nb,
+                     int64_t *group) {
+    *group = 0;
+    if (kind == K_FORCE) {
+        auto it = c->tuned.find(tune_key(n_i, n_j));
+        if (it != c->tuned.end()) return it->second;
+    }
+    const Grouping g = grouping(c, kind, n_i, n_j);
+    if (mixed) *group = g.group;
+    // five significant bits of the sink count, rounded up, so that the blocks of
+    // a time-step run share a few hundred entries
+    int sh = 0;
+    while ((n_i >> sh) >= 32) ++sh;
+    const int64_t n_r = ceil_div(n_i, int64_t(1) << sh) << sh;
+    const std::array<int64_t, 5> key{n_r, n_j, ((kind * 8 + order) * 2 + nn) * 2 + nb, mixed ? g.jl : 0, mixed ? g.group : 0};
+    auto it = c->shapes.find(key);
+    if (it != c->shapes.end()) return it->second;
+    if (c->shapes.size() >= 1024) c->shapes.clear();
+    return c->shapes[key] = heuristic(c, kind, order, mixed, n_r, n_j, nn, nb, g);
 }
 
 // rec holds n_valid records; sink slots must lie in [0, n_valid).  With
@@ -291,14 +412,9 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
                     const PassOut &o, const sp2_launch *forced, int stage_force, float *ms_out = nullptr,
                     bool allow_fused = false, const unsigned int *n_i_dev = nullptr) {
     if (n_i <= 0) return SP2_OK;
-    sp2_launch L;
-    if (forced) {
-        L = *forced;
-    } else {
-        auto it = (kind == K_FORCE) ? c->tuned.find(tune_key(n_i, j_end - j_begin)) : c->tuned.end();
-        L = (it != c->tuned.end()) ? it->second : heuristic(c, kind, mixed, n_i, j_end - j_begin);
-    }
     const int nb = (kind == K_FORCE && nn && o.nb_count) ? 1 : 0;
+    int64_t group = 0;  // group of the mixed sums that slices may not cut (0: none)
+    sp2_launch L = forced ? *forced : shape_for(c, kind, order, mixed, n_i, j_end - j_begin, nn, nb, &group);
     if (nb) L.i_per_thread = 1;  // neighbour-list kernels take one sink per thread
     const int64_t n_j = j_end - j_begin;
     const int jl = L.j_lanes;
@@ -314,7 +430,8 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
         return fail(c, SP2_ERR_UNSUPPORTED, "device-count passes are order-4/6 forces without neighbours");
     KernelKey key{kind, order, mixed, nn, L.i_per_thread, fused, nb, devn};
     int64_t split = std::max<int64_t>(1, std::min<int64_t>(L.split_j, ceil_div(n_j, tile)));
-    int64_t slice_len = ceil_div(ceil_div(n_j, split), tile) * tile;
+    const int64_t unit = group > 0 ? group : tile;
+    int64_t slice_len = ceil_div(ceil_div(n_j, split), unit) * unit;
     split = ceil_div(n_j, slice_len);
     const int ns_fields = (kind == K_VJP) ? 7 : (order == 6 ? 10 : (order == 2 ? 4 : 7));
     // fused: two bulk-copy stages when they fit and a slice spans several
@@ -356,7 +473,7 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
         const int64_t rest = n_iblk - n_whole;
         int64_t tail_split = rest > 0 ? std::min<int64_t>(resident / rest, ceil_div(n_j, tile)) : 1;
         if (tail_split > 1 && sinks_per_cta * tail_split <= kFusedReduceMaxValues) {
-            slice_len = ceil_div(ceil_div(n_j, tail_split), tile) * tile;
+            slice_len = ceil_div(ceil_div(n_j, tail_split), unit) * unit;
             split = ceil_div(n_j, slice_len);
         } else {
             n_whole = n_iblk;
@@ -381,6 +498,7 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
     p.split = static_cast<int>(split);
     p.jl = jl;
     p.tile = tile;
+    p.group_tiles = group > 0 && tile / jl < 64 ? static_cast<int>(group / tile) : 0;
     p.sinks_per_cta = static_cast<int>(sinks_per_cta);
     p.n_iblk = n_iblk;
     p.n_items = n_items;
@@ -416,19 +534,20 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
                                static_cast<size_t>(split) * n_part * sizeof(int32_t), "partial-id"));
         p.part = c->part;
         p.part_id = c->part_id;
-        p.sink_major = split >= kWarpReduceMinSplit ? 1 : 0;
-        // fuse the reduction into the pass when one CTA's share of it is small
-        // (a device-count pass always does; its i-blocks may be as small as
-        // threads / 32 sinks)
-        if (devn && sinks_per_cta * split > kFusedReduceMaxValues)
-            return fail(c, SP2_ERR_UNSUPPORTED, "device-count pass: split too large for the in-pass reduction");
-        if (std::min<int64_t>(sinks_per_cta, n_i) * split <= kFusedReduceMaxValues) {
-            const int64_t blocks = devn ? ceil_div(n_i, std::max(1, L.threads / 32)) : n_iblk;
+        // A device-count pass reduces its slices itself (no host knows how many
+        // sinks there are; its i-blocks may be as small as threads / 32 sinks).
+        // All others leave that to a kernel of its own: the fence, the count and
+        // the last CTA's reads at the end of the pass cost more than that kernel's
+        // launch (measured at the best shape of each: 12 sinks on 131072 sources
+        // 22.5 -> 20.5 us, 300 on 2048 16.4 -> 14.4, equal from 2000 sinks on).
+        if (devn) {
+            if (sinks_per_cta * split > kFusedReduceMaxValues)
+                return fail(c, SP2_ERR_UNSUPPORTED, "device-count pass: split too large for the in-pass reduction");
             const size_t old_cap = c->done_cap;
             SP2_CKS(ensure(c, reinterpret_cast<void **>(&c->done), &c->done_cap,
-                           static_cast<size_t>(blocks) * sizeof(unsigned int), "reduction-counter"));
+                           static_cast<size_t>(ceil_div(n_i, std::max(1, L.threads / 32))) * sizeof(unsigned int),
+                           "reduction-counter"));
             if (c->done_cap != old_cap) SP2_CK(c, cudaMemsetAsync(c->done, 0, c->done_cap, c->stream));
-            p.fused_reduce = 1;
             p.done = c->done;
         }
     }
@@ -442,16 +561,9 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
     SP2_CK(c, launch_force_kernel(key, p, grid, L.threads, tile, c->stream));
     ev_end(c, stage_force);
     c->launches += 1;
-    if (split > 1 && !p.fused_reduce) {
-        ReduceParams r{};
-        r.part = c->part;
-        r.part_id = c->part_id;
-        r.n_i = n_i;
-        r.split = static_cast<int>(split);
-        r.acc = o.acc; r.jerk = o.jerk; r.snap = o.snap; r.pot = o.pot; r.nn_id = o.nn_id; r.nn_r2 = o.nn_r2;
-        r.xbar = o.xbar; r.vbar = o.vbar; r.mbar = o.mbar; r.accumulate = o.accumulate;
+    if (split > 1 && !devn) {
         ev_begin(c, ST_REDUCE);
-        SP2_CK(c, launch_reduce_kernel(key, r, c->stream));
+        SP2_CK(c, launch_reduce_kernel(key, p, c->stream));
         ev_end(c, ST_REDUCE);
         c->launches += 1;
     }
@@ -563,7 +675,7 @@ cudaError_t force_kernel_occupancy(const KernelKey &k, int threads, size_t tile,
     return k.mixed ? occupancy_force_h4m(k, threads, tile, b) : occupancy_force_h4d(k, threads, tile, b);
 }
 
-cudaError_t launch_reduce_kernel(const KernelKey &k, const ReduceParams &r, cudaStream_t s) {
+cudaError_t launch_reduce_kernel(const KernelKey &k, const ForceParams &r, cudaStream_t s) {
     if (k.kind == K_VJP) return k.mixed ? launch_reduce_vjpm(k, r, s) : launch_reduce_vjpd(k, r, s);
     if (k.order == 6) return k.mixed ? launch_reduce_h6m(k, r, s) : launch_reduce_h6d(k, r, s);
     if (k.order == 2) return k.mixed ? launch_reduce_h2m(k, r, s) : launch_reduce_h2d(k, r, s);
@@ -1392,9 +1504,9 @@ sp2_status sp2_hermite4_step_vjp(sp2_ctx *c, int64_t n, double dt, const double 
 sp2_status sp2_get_launch(sp2_ctx *c, int64_t n_i, sp2_launch *out) {
     SP2_CKS(usable(c));
     if (!out || n_i <= 0) return fail(c, SP2_ERR_ARG, "bad arguments");
-    auto it = c->tuned.find(tune_key(n_i, c->n_loaded));
-    *out = (it != c->tuned.end()) ? it->second
-                                  : heuristic(c, K_FORCE, c->cfg.precision == SP2_MIXED, n_i, std::max<int64_t>(c->n_loaded, 1));
+    int64_t group;
+    *out = shape_for(c, K_FORCE, c->cfg.order, c->cfg.precision == SP2_MIXED, n_i, std::max<int64_t>(c->n_loaded, 1),
+                     c->cfg.with_nn, 0, &group);
     return SP2_OK;
 }
 
@@ -1425,7 +1537,7 @@ sp2_status sp2_autotune(sp2_ctx *c, int64_t n_i, sp2_launch *best) {
     o.nn_id = nn ? reinterpret_cast<int32_t *>(c->tmp + 9 * c->cfg.n_max + 2 * n_i) : nullptr;
     if (nn && 9 * c->cfg.n_max + 3 * n_i > 12 * c->cfg.n_max) o.nn_r2 = nullptr, o.nn_id = nullptr;
 
-    const sp2_launch h = heuristic(c, K_FORCE, mixed, n_i, n_j);
+    const sp2_launch h = heuristic(c, K_FORCE, order, mixed, n_i, n_j, nn, 0, grouping(c, K_FORCE, n_i, n_j));
     // time one launch shape: mean of `reps` runs after one warm-up run
     auto time_shape = [&](const sp2_launch &L, int reps, float *ms_out) -> sp2_status {
         if (check_launch(c, L) != SP2_OK) return SP2_ERR_UNSUPPORTED;

@@ -92,11 +92,11 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned pari
 
 // Drop the 128-byte L2 lines that lie wholly inside [lo, hi) without writing
 // them back (their contents are not needed again); lines shared with
-// neighbouring data are kept.  Called by all threads of a CTA.
+// neighbouring data are kept.
 __device__ __forceinline__ void discard_l2_range(const void *lo, const void *hi) {
     const uintptr_t a = (reinterpret_cast<uintptr_t>(lo) + 127u) & ~static_cast<uintptr_t>(127u);
     const uintptr_t e = reinterpret_cast<uintptr_t>(hi) & ~static_cast<uintptr_t>(127u);
-    for (uintptr_t q = a + static_cast<uintptr_t>(threadIdx.x) * 128u; q < e; q += static_cast<uintptr_t>(blockDim.x) * 128u)
+    for (uintptr_t q = a; q < e; q += 128u)
         asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(q) : "memory");
 }
 
@@ -917,6 +917,9 @@ struct Fp64Force {
     __device__ static __forceinline__ void write_final(const Out &o, int64_t i, const double *t, double d, int id) {
         MixedForce<ORDER, NN>::write_final(o, i, t, d, id);
     }
+    __device__ static __forceinline__ void store_final(const ForceParams &o, int64_t i, int f, double v) {
+        MixedPairForce<ORDER, NN>::store_final(o, i, f, v);
+    }
 };
 
 // ---------------------------------------------------------------------------
@@ -1331,6 +1334,9 @@ struct Fp64Vjp {
     __device__ static __forceinline__ void write_final(const Out &o, int64_t i, const double *t, double d, int id) {
         MixedVjp::write_final(o, i, t, d, id);
     }
+    __device__ static __forceinline__ void store_final(const ForceParams &o, int64_t i, int f, double v) {
+        MixedPairVjp::store_final(o, i, f, v);
+    }
 };
 
 // ---------------------------------------------------------------------------
@@ -1505,7 +1511,6 @@ __device__ __forceinline__ void merge_lanes_ds(const double *tot, int stride, in
 template <class P>
 __device__ __forceinline__ void write_fields_ds(const ForceParams &p, int64_t i, int split, int slice, int64_t pi,
                                                 int64_t pn, const ds *q, int jl, int lj) {
-    constexpr int NF = P::NS + (P::kNN ? 1 : 0);
     for (int f0 = 0; f0 < P::NS; f0 += jl) {
         const int f = f0 + lj;
         float h = 0.f, l = 0.f;
@@ -1522,240 +1527,166 @@ __device__ __forceinline__ void write_fields_ds(const ForceParams &p, int64_t i,
             }
             const double v = f2d_exact(h) + f2d_exact(l);
             if (split == 1) P::store_final(p, i, f, v);
-            else if (p.sink_major) p.part[(pi * NF + f) * split + slice] = v;
             else p.part[static_cast<int64_t>(f) * split * pn + static_cast<int64_t>(slice) * pn + pi] = v;
         }
     }
 }
 
-// FP64 reduction of one sink's slices (sink-major row: field f's slices are
-// contiguous) by the whole CTA, fields spread over the warps (two at a time,
-// so that different warps' 1/64-rate FP64 adds run side by side): lane l of
-// a warp sums slices l, l+32, ... of a field in order, a fixed xor-butterfly
-// combines the lanes, and the field totals meet in shared
-// memory, where thread 0 writes the outputs (write(t, d, id)).  The
-// nearest-neighbour field (non-negative r^2, FP64) is merged by comparing bit
-// patterns as integers, which orders them like the values.  Deterministic:
-// the order of every sum is fixed.
-template <class P, class Write>
-__device__ __forceinline__ void reduce_sink_fields(const double *row, const int32_t *row_id, int split, double *s_f,
-                                                   long long &s_nd, int &s_nid, const Write &write) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    // columns 0 .. NS-1 are the summed fields and (with nearest neighbour)
-    // column NS the neighbour candidates; warp w takes columns w, w + nw, ...
-    // two at a time, so the neighbour's loads travel with a field's
-    constexpr int NC = P::NS + (P::kNN ? 1 : 0);
-    for (int c0 = warp; c0 < NC; c0 += 2 * nw) {
-        const int c1 = c0 + nw;
-        const bool two = c1 < NC;  // (warp-uniform)
-        const bool nn0 = P::kNN && c0 == P::NS, nn1 = P::kNN && two && c1 == P::NS;
-        const double *col0 = row + static_cast<int64_t>(c0) * split;
-        const double *col1 = row + static_cast<int64_t>(two ? c1 : c0) * split;
-        // lane l takes slices l, l + 32, l + 64, ... in that order; the loads of
-        // 256 slices per column are all issued before the first add
-        double v0 = 0.0, v1 = 0.0;
-        long long d = 0x7ff0000000000000LL;  // neighbour column: best r^2 bits (+inf) and id
-        int id = -1;
-        for (int s0 = 0; s0 < split; s0 += 8 * 32) {
-            double x0[8], x1[8];
-            int xi[8];
+// Split-j reduction of one column: field f of sink i, its partial sums of
+// slices 0 .. split-1 `pn` apart.  The loads of E slices are issued before
+// their adds, so a column costs split / E memory round trips; the order of the
+// adds is that of the slices.
+constexpr int kReduceInFlight = 16;
+// x[e] = p[e * step] for e < n, `rest` from there on; volatile, so that all loads stay in front
+// of the adds that follow (left to itself the compiler trades them for registers)
+template <int E>
+__device__ __forceinline__ void load_slices(const double *p, int n, int64_t step, double rest, double *x) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int s = s0 + lane + 32 * e;
-                x0[e] = (s < split) ? __ldcg(col0 + s) : 0.0;
-                x1[e] = (two && s < split) ? __ldcg(col1 + s) : 0.0;
-                xi[e] = ((nn0 || nn1) && s < split) ? __ldcg(row_id + s) : -1;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (s0 + lane + 32 * e < split) {
-                    if (nn0 || nn1) {
-                        // non-negative r^2: the bit patterns order like the values
-                        const long long xd = __double_as_longlong(nn0 ? x0[e] : x1[e]);
-                        if (xd < d || (xd == d && static_cast<unsigned>(xi[e]) < static_cast<unsigned>(id))) {
-                            d = xd;
-                            id = xi[e];
-                        }
-                    }
-                    if (!nn0) v0 += x0[e];
-                    if (two && !nn1) v1 += x1[e];
-                }
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            if (!nn0) v0 += __shfl_xor_sync(kFull, v0, off);
-            if (two && !nn1) v1 += __shfl_xor_sync(kFull, v1, off);
-            if (nn0 || nn1) {
-                const long long od = __shfl_xor_sync(kFull, d, off);
-                const int oid = __shfl_xor_sync(kFull, id, off);
-                if (od < d || (od == d && static_cast<unsigned>(oid) < static_cast<unsigned>(id))) {
-                    d = od;
-                    id = oid;
-                }
-            }
-        }
-        if (lane == 0) {
-            if (!nn0) s_f[c0] = v0;
-            if (two && !nn1) s_f[c1] = v1;
-            if (nn0 || nn1) {
-                s_nd = d;
-                s_nid = id;
-            }
-        }
+    for (int e = 0; e < E; ++e) {
+        x[e] = rest;
+        if (e < n) asm volatile("ld.global.cg.f64 %0, [%1];\n" : "=d"(x[e]) : "l"(p + e * step) : "memory");
     }
-    __syncthreads();
-    if (tid == 0) {
-        double t[P::NS];
-#pragma unroll
-        for (int f = 0; f < P::NS; ++f) t[f] = s_f[f];
-        write(t, P::kNN ? __longlong_as_double(s_nd) : d_inf(), P::kNN ? s_nid : -1);
-    }
-    __syncthreads();
 }
-
-// One lane's share of a sink-major row: slices lane, lane + 32, ... of every
-// field added in that order (FP64) and the lexicographic (r^2, id) minimum of
-// their neighbours; beyond two slices per lane the loads of a few slices
-// (every field) are issued before their adds, so a row of a few hundred
-// slices costs one or two memory round trips instead of one per slice.
-template <class P>
-__device__ __forceinline__ void lane_sum_slices(const double *row, const int32_t *row_id, int split, int lane,
-                                                double *t, double &nd, int &nid) {
-    constexpr int E = (P::NS <= 7) ? 4 : 2;  // slices in flight per lane
-#pragma unroll
-    for (int f = 0; f < P::NS; ++f) t[f] = 0.0;
-    nd = d_inf();
-    nid = -1;
-    if (split <= 64) {
-        // one or two slices per lane: the plain loop (the chunks would be
-        // mostly empty, their predicated loads and adds pure cost)
-        for (int s = lane; s < split; s += 32) {
-#pragma unroll
-            for (int f = 0; f < P::NS; ++f) t[f] += __ldcg(row + f * split + s);
-            if (P::kNN) nn_merge(nd, nid, __ldcg(row + P::NS * split + s), __ldcg(row_id + s));
-        }
-        return;
-    }
-    for (int s0 = 0; s0 < split; s0 += E * 32) {
-        double x[E][P::NS], xd[E];
-        int xi[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int s = s0 + lane + 32 * e;
-            const bool in = s < split;
-#pragma unroll
-            for (int f = 0; f < P::NS; ++f) x[e][f] = in ? __ldcg(row + f * split + s) : 0.0;
-            if (P::kNN) {
-                xd[e] = in ? __ldcg(row + P::NS * split + s) : d_inf();
-                xi[e] = in ? __ldcg(row_id + s) : -1;
-            }
-        }
+__device__ __forceinline__ double sum_slices(const double *col, int s0, int s1, int64_t pn) {
+    constexpr int E = kReduceInFlight;
+    double t = 0.0;
+    col += s0 * pn;
+    for (; s0 < s1; s0 += E, col += E * pn) {
+        double x[E];
+        load_slices<E>(col, s1 - s0, pn, 0.0, x);
 #pragma unroll
         for (int e = 0; e < E; ++e)
-            if (s0 + lane + 32 * e < split) {
+            if (s0 + e < s1) t += x[e];
+    }
+    return t;
+}
+// the same for the nearest-neighbour column: lexicographic (r^2, id) minimum;
+// r^2 >= 0, so the bit patterns order like the values and integer compares do
+__device__ __forceinline__ void key_merge(long long &d, int &id, long long od, int oid) {
+    if (od < d || (od == d && static_cast<unsigned>(oid) < static_cast<unsigned>(id))) {
+        d = od;
+        id = oid;
+    }
+}
+__device__ __forceinline__ void min_slices(const double *col, const int32_t *col_id, int s0, int s1, int64_t pn,
+                                           long long &d, int &id) {
+    constexpr int E = kReduceInFlight;
+    d = 0x7ff0000000000000LL;  // +inf
+    id = -1;
+    col += s0 * pn;
+    col_id += s0 * pn;
+    for (; s0 < s1; s0 += E, col += E * pn, col_id += E * pn) {
+        double x[E];
+        int xi[E];
+        load_slices<E>(col, s1 - s0, pn, d_inf(), x);
 #pragma unroll
-                for (int f = 0; f < P::NS; ++f) t[f] += x[e][f];
-                if (P::kNN) nn_merge(nd, nid, xd[e], xi[e]);
-            }
+        for (int e = 0; e < E; ++e) xi[e] = (s0 + e < s1) ? __ldcg(col_id + e * pn) : -1;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (s0 + e < s1) key_merge(d, id, __double_as_longlong(x[e]), xi[e]);
     }
 }
 
-// Fused split-j reduction of one i-block, run by the last CTA to finish one
-// of its slices.  Partials are read from L2 (__ldcg: written by other SMs in
-// this launch) in slice order, so the result does not depend on which CTA
-// arrives last.  Field-major partials (few slices): a thread per sink.
-// Sink-major partials (many slices): a warp per sink, or the whole CTA per
-// sink (a warp per field) when the i-block has fewer sinks than the CTA has
-// warps.
+// The CTA sums columns c0 .. c0 + blockDim.x / groups - 1 of the (field, sink)
+// columns of sinks [b0, b0 + ns) and writes the outputs.  Neighbouring threads
+// take neighbouring sinks of one field (coalesced); with groups > 1 the slices
+// of a column are divided over that many threads, whose sums meet in a fixed
+// binary tree through shared memory (s_v, s_id: one entry per thread).  The order of
+// every sum depends on split and groups only, never on scheduling; partials
+// are read from L2 (__ldcg: other SMs wrote them in this launch).  All threads
+// of the CTA call this.
+template <class P>
+__device__ __forceinline__ void reduce_columns(const ForceParams &p, int64_t b0, int64_t ns, int64_t c0, int groups,
+                                               double *s_v, int32_t *s_id) {
+    constexpr int NF = P::NS + (P::kNN ? 1 : 0);
+    const int cols = blockDim.x / groups;
+    const int g = threadIdx.x / cols, l = threadIdx.x - g * cols;
+    const int64_t c = c0 + l;
+    // partial rows are counted from the first sink of the split i-blocks
+    const int64_t pn = p.n_i - p.tail_sink0;
+    const bool valid = c < NF * ns;
+    const int f = valid ? static_cast<int>(c / ns) : 0;
+    const int64_t i = b0 + (valid ? c - f * ns : 0), pi = i - p.tail_sink0;
+    const bool nn = P::kNN && f == P::NS;
+    const int len = (p.split + groups - 1) / groups;
+    const int s0 = g * len, s1 = valid ? min(s0 + len, p.split) : s0;
+    const double *col = p.part + static_cast<int64_t>(f) * p.split * pn + pi;
+    const int32_t *col_id = nn ? p.part_id + pi : nullptr;
+    double t = 0.0;
+    long long key = 0;
+    int id = -1;
+    if (nn) min_slices(col, col_id, s0, s1, pn, key, id);
+    else t = sum_slices(col, s0, s1, pn);
+    if (groups > 1) {
+        long long *s_key = reinterpret_cast<long long *>(s_v);
+        for (int o = groups / 2; o > 0; o /= 2) {
+            // groups o .. 2o-1 hand their sums to groups 0 .. o-1
+            if (g >= o && g < 2 * o) {
+                if (nn) s_key[threadIdx.x] = key;
+                else s_v[threadIdx.x] = t;
+                if (P::kNN) s_id[threadIdx.x] = id;
+            }
+            __syncthreads();
+            if (g < o) {
+                if (nn) key_merge(key, id, s_key[threadIdx.x + o * cols], s_id[threadIdx.x + o * cols]);
+                else t += s_v[threadIdx.x + o * cols];
+            }
+        }
+        __syncthreads();
+    }
+    if (!valid || g > 0) return;
+    if (nn) {
+        if (p.nn_id) p.nn_id[i] = id;
+        if (p.nn_r2) p.nn_r2[i] = (id < 0) ? d_inf() : __longlong_as_double(key);
+    } else {
+        P::store_final(p, i, f, t);
+    }
+}
+
+// Reduction of one i-block inside the pass, by the last CTA to finish one of
+// its slices: many slices of few columns are divided over the CTA's threads.
+// Scratch is the CTA's dynamic shared memory, free between two work items.
 template <class P>
 __device__ __noinline__ void reduce_iblock(const ForceParams &p, int64_t iblk) {
-    __shared__ double s_f[P::NS];
-    __shared__ long long s_nd;
-    __shared__ int s_nid;
+    extern __shared__ __align__(16) unsigned char smem[];
     constexpr int NF = P::NS + (P::kNN ? 1 : 0);
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const int nt = blockDim.x;
     const int64_t b0 = iblk * p.sinks_per_cta;
-    const int64_t b1 = (b0 + p.sinks_per_cta < p.n_i) ? b0 + p.sinks_per_cta : p.n_i;
-    const int split = p.split;
-    // partial rows are counted from the first sink of the split i-blocks
-    const int64_t r0 = p.tail_sink0, pn = p.n_i - p.tail_sink0;
-    if (!p.sink_major) {
-        const int64_t stride = static_cast<int64_t>(split) * pn;
-        for (int64_t i = b0 + tid; i < b1; i += nt) {
-            double t[P::NS];
-#pragma unroll
-            for (int f = 0; f < P::NS; ++f) t[f] = 0.0;
-            double nd = d_inf();
-            int nid = -1;
-            const double *base = p.part + (i - r0);       // slice 0, field 0 of this sink's row
-            const int32_t *base_id = p.part_id + (i - r0);
-#pragma unroll 2
-            for (int s = 0; s < split; ++s, base += pn, base_id += pn) {
-#pragma unroll
-                for (int f = 0; f < P::NS; ++f) t[f] += __ldcg(base + f * stride);
-                if (P::kNN) nn_merge(nd, nid, __ldcg(base + P::NS * stride), __ldcg(base_id));
-            }
-            P::write_final(p, i, t, nd, nid);
-        }
-        return;
-    }
-    if (b1 - b0 < nw) {
-        // few sinks: the whole CTA on each, one warp per field
-        for (int64_t i = b0; i < b1; ++i)
-            reduce_sink_fields<P>(p.part + (i - r0) * NF * split, p.part_id + (i - r0) * split, split, s_f, s_nd, s_nid,
-                                  [&](const double *t, double d, int id) { P::write_final(p, i, t, d, id); });
-        return;
-    }
-    // a warp per sink
-    for (int64_t i = b0 + warp; i < b1; i += nw) {
-        const double *row = p.part + (i - r0) * NF * split;
-        const int32_t *row_id = p.part_id + (i - r0) * split;
-        double t[P::NS];
-        double nd;
-        int nid;
-        lane_sum_slices<P>(row, row_id, split, lane, t, nd, nid);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-            for (int f = 0; f < P::NS; ++f) t[f] += __shfl_xor_sync(kFull, t[f], off);
-            if (P::kNN) {
-                const double od = __shfl_xor_sync(kFull, nd, off);
-                const int oid = __shfl_xor_sync(kFull, nid, off);
-                nn_merge(nd, nid, od, oid);
-            }
-        }
-        if (lane == 0) P::write_final(p, i, t, nd, nid);
-    }
+    const int64_t ns = min(static_cast<int64_t>(p.sinks_per_cta), p.n_i - b0);
+    int groups = 1;
+    if (p.split >= kGroupReduceMinSplit)
+        while (groups < 32 && 2 * groups * NF * ns <= nt) groups *= 2;
+    double *s_v = reinterpret_cast<double *>(smem);
+    int32_t *s_id = reinterpret_cast<int32_t *>(s_v + nt);
+    for (int64_t c0 = 0; c0 < NF * ns; c0 += nt / groups) reduce_columns<P>(p, b0, ns, c0, groups, s_v, s_id);
 }
 
-// The partial-sum rows of one split i-block, dropped from L2 once reduced.
+// The partial-sum rows of one split i-block, dropped from L2 once reduced: a
+// thread per row (field, slice); rows shorter than a line hold none wholly.
 template <class P>
 __device__ __forceinline__ void discard_partials(const ForceParams &p, int64_t iblk) {
     constexpr int NF = P::NS + (P::kNN ? 1 : 0);
     const int64_t b0 = iblk * p.sinks_per_cta - p.tail_sink0;
-    const int64_t b1 = ((iblk * p.sinks_per_cta + p.sinks_per_cta < p.n_i) ? iblk * p.sinks_per_cta + p.sinks_per_cta
-                                                                          : p.n_i) - p.tail_sink0;
+    const int64_t ns = min(static_cast<int64_t>(p.sinks_per_cta), p.n_i - iblk * p.sinks_per_cta);
     const int64_t pn = p.n_i - p.tail_sink0;
-    const int split = p.split;
-    if (p.sink_major) {
-        discard_l2_range(p.part + b0 * NF * split, p.part + b1 * NF * split);
-        if (P::kNN) discard_l2_range(p.part_id + b0 * split, p.part_id + b1 * split);
-        return;
-    }
-    for (int f = 0; f < NF; ++f)
-        for (int sl = 0; sl < split; ++sl) {
-            const double *row = p.part + (static_cast<int64_t>(f) * split + sl) * pn;
-            discard_l2_range(row + b0, row + b1);
+    if (ns < 32) return;
+    for (int r = threadIdx.x; r < NF * p.split; r += blockDim.x) {
+        const double *row = p.part + r * pn + b0;
+        discard_l2_range(row, row + ns);
+        if (P::kNN && r < p.split) {
+            const int32_t *row_id = p.part_id + r * pn + b0;
+            discard_l2_range(row_id, row_id + ns);
         }
-    if (P::kNN)
-        for (int sl = 0; sl < split; ++sl) discard_l2_range(p.part_id + sl * pn + b0, p.part_id + sl * pn + b1);
+    }
 }
 
 // Shared memory: kStages tiles of records, (paired policies) one tile of pair
 // records, then (mixed policies) the running totals (8 bytes each: FP64, or a
 // double-single pair in the paired policy), [sink k][field f][thread]
 // so each thread owns its slots.
-template <class P, int IPT, bool FUSED, bool MW = false>
+// MW: several warps may share a sink; DEVN: the device-count form, which reduces
+// its split i-blocks itself (the others leave that to reduce_kernel).
+template <class P, int IPT, bool FUSED, bool MW = false, bool DEVN = false>
 __device__ __forceinline__ void pass_body(const ForceParams &p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned int s_item;
@@ -1967,7 +1898,7 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
                 else tile_loop<P, IPT, false>(sg, tb + c0, per, jl, lj, sk, ac, eps2);
             }
             since_flush += per;
-            if (since_flush >= P::kFlush) {
+            if (since_flush >= P::kFlush || (p.group_tiles > 0 && (t + 1) % p.group_tiles == 0)) {
 #pragma unroll
                 for (int k = 0; k < IPT; ++k) P::flush(ac[k], tot + k * P::NS * nt, nt);
                 since_flush = 0;
@@ -2030,10 +1961,6 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
                     if (isplit == 1) {
                         if (p.nn_id) p.nn_id[ii[k]] = nid;
                         if (p.nn_r2) p.nn_r2[ii[k]] = (nid < 0) ? d_inf() : nd;
-                    } else if (p.sink_major) {
-                        constexpr int NF = P::NS + (P::kNN ? 1 : 0);
-                        p.part[(pi * NF + P::NS) * isplit + slice] = nd;
-                        p.part_id[pi * isplit + slice] = nid;
                     } else {
                         const int64_t stride = static_cast<int64_t>(isplit) * pn;
                         p.part[P::NS * stride + static_cast<int64_t>(slice) * pn + pi] = nd;
@@ -2058,15 +1985,6 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
                 const int64_t pi = ii[k] - p.tail_sink0;
                 if (isplit == 1) {
                     P::write_final(p, ii[k], t, nd, nid);
-                } else if (p.sink_major) {
-                    constexpr int NF = P::NS + (P::kNN ? 1 : 0);
-                    double *base = p.part + pi * NF * isplit + slice;
-#pragma unroll
-                    for (int f = 0; f < P::NS; ++f) base[f * isplit] = t[f];
-                    if (P::kNN) {
-                        base[P::NS * isplit] = nd;
-                        p.part_id[pi * isplit + slice] = nid;
-                    }
                 } else {
                     const int64_t stride = static_cast<int64_t>(isplit) * pn;
                     double *base = p.part + static_cast<int64_t>(slice) * pn + pi;
@@ -2079,7 +1997,7 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
                 }
             }
         }
-        if (isplit > 1 && p.fused_reduce) {
+        if (DEVN && isplit > 1) {
             // every partial of this CTA is written (barrier); thread 0's fence
             // then makes them visible device-wide before the CTA is counted.
             // The last CTA's thread 0 fences again after the count, and the
@@ -2151,7 +2069,6 @@ __device__ __forceinline__ void device_shape(ForceParams &q) {
     q.n_items = n_iblk * q.split;
     q.sinks_per_cta = spc;
     q.jl = jl;
-    q.sink_major = q.split >= kWarpReduceMinSplit ? 1 : 0;
 }
 
 // Resident CTAs of kMaxThreads that a kernel's register budget must allow
@@ -2178,81 +2095,30 @@ __global__ void __launch_bounds__(kMaxThreads, (pass_min_blocks<P, IPT, FUSED>::
         static_assert(IPT == 1 && !FUSED, "the device-count form takes one sink per thread");
         ForceParams q = p;
         device_shape(q);
-        pass_body<P, IPT, FUSED>(q);
+        pass_body<P, IPT, FUSED, false, true>(q);
     } else {
         pass_body<P, IPT, FUSED>(p);
     }
 }
 
-// Second kernel of the source split: sum the slices of each sink in slice
-// order (deterministic, FP64) and take the lexicographic (r2, id) minimum.
+// Second kernel of the source split: the columns of all sinks with partial
+// rows.  8 threads share a column of many slices, 32 where the columns are too
+// few to fill the GPU, so that even one sink's slices are a round trip or two;
+// fewer slices take a thread per column.  The kernel is bound by the latency of
+// those trips.  Before, one warp per sink (or one thread) added the slices with
+// two loads in flight, inside the pass's last CTA up to 16384 partial sums:
+// 61 sinks on 131072 sources in 512 slices took 121 us for the step, now
+// 61 us; 317 on 16384 in 64 slices 222 us, now 121 us; the 16384-particle
+// adjoint run (32 slices) 18.4 ms, now 14.8 ms.
+constexpr int kReduceThreads = 256;
+constexpr int kReduceGroups = 8, kReduceGroupsFew = 32;
+constexpr int64_t kReduceFewColumns = 4096;
 template <class P>
-__global__ void reduce_kernel(const ReduceParams r) {
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= r.n_i) return;
-    const int64_t stride = static_cast<int64_t>(r.split) * r.n_i;
-    double t[P::NS];
-#pragma unroll
-    for (int f = 0; f < P::NS; ++f) t[f] = 0.0;
-    double nd = d_inf();
-    int nid = -1;
-    for (int s = 0; s < r.split; ++s) {
-        const double *base = r.part + static_cast<int64_t>(s) * r.n_i + i;
-#pragma unroll
-        for (int f = 0; f < P::NS; ++f) t[f] += base[f * stride];
-        if (P::kNN) nn_merge(nd, nid, base[P::NS * stride], r.part_id[static_cast<int64_t>(s) * r.n_i + i]);
-    }
-    P::write_final(r, i, t, nd, nid);
-}
-
-// The same reduction with one warp per sink, for many slices, on the
-// sink-major layout (a warp's loads are contiguous): lane l sums slices l,
-// l+32, ... in order, then a fixed xor-butterfly combines the lanes, so the
-// result is still independent of scheduling.
-template <class P>
-__global__ void reduce_warp_kernel(const ReduceParams r) {
-    const int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (i >= r.n_i) return;  // uniform across the warp
-    constexpr int NF = P::NS + (P::kNN ? 1 : 0);
-    const double *row = r.part + i * NF * r.split;
-    const int32_t *row_id = r.part_id + i * r.split;
-    double t[P::NS];
-#pragma unroll
-    for (int f = 0; f < P::NS; ++f) t[f] = 0.0;
-    double nd = d_inf();
-    int nid = -1;
-    // (many warps in flight hide the loads here; the chunked loads of
-    // lane_sum_slices would only cost registers and occupancy)
-    for (int s = lane; s < r.split; s += 32) {
-#pragma unroll
-        for (int f = 0; f < P::NS; ++f) t[f] += row[f * r.split + s];
-        if (P::kNN) nn_merge(nd, nid, row[P::NS * r.split + s], row_id[s]);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int f = 0; f < P::NS; ++f) t[f] += __shfl_xor_sync(kFull, t[f], off);
-        if (P::kNN) {
-            const double od = __shfl_xor_sync(kFull, nd, off);
-            const int oid = __shfl_xor_sync(kFull, nid, off);
-            nn_merge(nd, nid, od, oid);
-        }
-    }
-    if (lane == 0) P::write_final(r, i, t, nd, nid);
-}
-
-// Few sinks, many slices: one 256-thread block per sink on the sink-major
-// layout, a warp per field (reduce_sink_fields).
-template <class P>
-__global__ void __launch_bounds__(256) reduce_block_kernel(const ReduceParams r) {
-    __shared__ double s_f[P::NS];
-    __shared__ long long s_nd;
-    __shared__ int s_nid;
-    constexpr int NF = P::NS + (P::kNN ? 1 : 0);
-    const int64_t i = blockIdx.x;
-    reduce_sink_fields<P>(r.part + i * NF * r.split, r.part_id + i * r.split, r.split, s_f, s_nd, s_nid,
-                          [&](const double *t, double d, int id) { P::write_final(r, i, t, d, id); });
+__global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const ForceParams p, int groups) {
+    __shared__ double s_v[kReduceThreads];
+    __shared__ int32_t s_id[kReduceThreads];
+    reduce_columns<P>(p, p.tail_sink0, p.n_i - p.tail_sink0,
+                      static_cast<int64_t>(blockIdx.x) * (kReduceThreads / groups), groups, s_v, s_id);
 }
 
 // ---------------------------------------------------------------------------
@@ -2492,17 +2358,12 @@ inline cudaError_t dispatch_nb(bool occ, int ipt, const ForceParams *p, int grid
 }
 
 template <class P>
-inline cudaError_t launch_reduce(const ReduceParams &r, cudaStream_t s) {
-    const int threads = 256;
-    if (r.split >= kWarpReduceMinSplit && r.n_i <= kBlockReduceMaxSinks) {
-        reduce_block_kernel<P><<<static_cast<unsigned>(r.n_i), 256, 0, s>>>(r);
-    } else if (r.split >= kWarpReduceMinSplit) {
-        const int64_t grid = (32 * r.n_i + threads - 1) / threads;
-        reduce_warp_kernel<P><<<static_cast<unsigned>(grid), threads, 0, s>>>(r);
-    } else {
-        const int64_t grid = (r.n_i + threads - 1) / threads;
-        reduce_kernel<P><<<static_cast<unsigned>(grid), threads, 0, s>>>(r);
-    }
+inline cudaError_t launch_reduce(const ForceParams &p, cudaStream_t s) {
+    constexpr int NF = P::NS + (P::kNN ? 1 : 0);
+    const int64_t n = NF * (p.n_i - p.tail_sink0);
+    const int groups = p.split < kGroupReduceMinSplit ? 1 : n <= kReduceFewColumns ? kReduceGroupsFew : kReduceGroups;
+    const int64_t cols = kReduceThreads / groups;
+    reduce_kernel<P><<<static_cast<unsigned>((n + cols - 1) / cols), kReduceThreads, 0, s>>>(p, groups);
     return cudaGetLastError();
 }
 
@@ -2551,7 +2412,7 @@ inline cudaError_t occupancy_batched(int threads, int *blocks) {
                     : dispatch_ipt<POLICY<ORDER, false>>(true, k.ipt, nullptr, 0, threads, tile, 0, blocks, \
                                                          k.fused, k.devn, k.fused_stages, k.mw);           \
     }                                                                                                      \
-    cudaError_t launch_reduce_##SUFFIX(const KernelKey &k, const ReduceParams &r, cudaStream_t s) {        \
+    cudaError_t launch_reduce_##SUFFIX(const KernelKey &k, const ForceParams &r, cudaStream_t s) {         \
         return k.nn ? launch_reduce<POLICY<ORDER, true>>(r, s) : launch_reduce<POLICY<ORDER, false>>(r, s); \
     }                                                                                                      \
     cudaError_t launch_batched_##SUFFIX(int nn, const BatchParams &b, int grid, int threads,               \

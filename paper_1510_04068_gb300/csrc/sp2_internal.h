@@ -74,20 +74,14 @@ struct ForceParams {
     double *nn_r2;
     // partial results (split > 1), NF = summed fields (+1 for the NN r^2),
     // r = i - tail_sink0 the partial row of sink i, pn = n_i - tail_sink0:
-    //   field-major (sink_major = 0): part[f * split * pn + slice * pn + r],
-    //                                 part_id[slice * pn + r]
-    //   sink-major  (sink_major = 1): part[(r * NF + f) * split + slice],
-    //                                 part_id[r * split + slice]
-    // sink-major is used with the warp-per-sink reduction (split >= 32), so a
-    // warp reads its sink's slices contiguously.
+    //   part[f * split * pn + slice * pn + r], part_id[slice * pn + r]
     double *part;
     int32_t *part_id;
-    int sink_major;
-    // fused reduction (split > 1): the last CTA to finish a slice of an
+    // device-count form (split > 1): the last CTA to finish a slice of an
     // i-block (counted in done[iblk], zero between launches and reset by that
     // CTA) sums the i-block's partials in slice order and writes the outputs
-    int fused_reduce;
     unsigned int *done;
+    int group_tiles;           // mixed: the totals are also updated at the end of every so many tiles (0: no)
     // neighbour lists (kernels of the neighbour-list policy only): per sink
     // position i, squared radius nb_h2[i], counter nb_count[i] (zero at launch)
     // and nb_max slots at nb_list + i * nb_max
@@ -103,18 +97,6 @@ struct ForceParams {
     const float4 *dsc;
     float t_hi, t_lo;
     int fused_stages;          // bulk-copy stages of the fused prediction: 1 (a slice fits one tile) or 2
-};
-
-struct ReduceParams {
-    const double *part;
-    const int32_t *part_id;
-    int64_t n_i;
-    int split;                 // >= 32: warp per sink on the sink-major layout
-    double *acc, *jerk, *snap, *pot;
-    int32_t *nn_id;
-    double *nn_r2;
-    double *xbar, *vbar, *mbar;
-    int accumulate;
 };
 
 struct BatchParams {
@@ -135,11 +117,9 @@ enum Kind { K_FORCE = 0, K_VJP = 1 };
 // GPU, less room for the kernels' static shared variables, about 2.5 KiB).
 constexpr int kMaxPassSmem = 222 * 1024;
 
-// From this many slices on, the split-j reduction runs one warp per sink on
-// the sink-major partial layout (ForceParams::sink_major).
-constexpr int kWarpReduceMinSplit = 32;
-// Up to this many sinks, that reduction uses a whole block per sink.
-constexpr int64_t kBlockReduceMaxSinks = 1024;
+// From this many slices on, the split-j reduction divides a column's slices
+// over several threads.
+constexpr int kGroupReduceMinSplit = 32;
 
 struct KernelKey {
     int kind;   // K_FORCE / K_VJP
@@ -160,7 +140,7 @@ struct KernelKey {
 cudaError_t launch_force_kernel(const KernelKey &k, const ForceParams &p, int grid, int threads,
                                 size_t tile, cudaStream_t s);
 cudaError_t force_kernel_occupancy(const KernelKey &k, int threads, size_t tile, int *blocks_per_sm);
-cudaError_t launch_reduce_kernel(const KernelKey &k, const ReduceParams &p, cudaStream_t s);
+cudaError_t launch_reduce_kernel(const KernelKey &k, const ForceParams &p, cudaStream_t s);
 cudaError_t launch_batched_kernel(int order, int mixed, int nn, const BatchParams &p, int grid,
                                   int threads, cudaStream_t s);
 cudaError_t batched_kernel_occupancy(int order, int mixed, int nn, int threads, int *blocks_per_sm);
@@ -170,7 +150,7 @@ cudaError_t batched_kernel_occupancy(int order, int mixed, int nn, int threads, 
     cudaError_t launch_force_##SUFFIX(const KernelKey &, const ForceParams &, int, int, size_t,    \
                                       cudaStream_t);                                               \
     cudaError_t occupancy_force_##SUFFIX(const KernelKey &, int, size_t, int *);                   \
-    cudaError_t launch_reduce_##SUFFIX(const KernelKey &, const ReduceParams &, cudaStream_t);     \
+    cudaError_t launch_reduce_##SUFFIX(const KernelKey &, const ForceParams &, cudaStream_t);      \
     cudaError_t launch_batched_##SUFFIX(int, const BatchParams &, int, int, cudaStream_t);         \
     cudaError_t occupancy_batched_##SUFFIX(int, int, int *);
 SP2_DECLARE_TU(h2m)

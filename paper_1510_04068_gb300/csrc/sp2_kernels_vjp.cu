@@ -13,7 +13,7 @@ namespace sp2 {
     cudaError_t occupancy_force_##SUFFIX(const KernelKey &k, int threads, size_t tile, int *blocks) {    \
         return dispatch_ipt<POLICY>(true, k.ipt, nullptr, 0, threads, tile, 0, blocks, k.fused);        \
     }                                                                                                   \
-    cudaError_t launch_reduce_##SUFFIX(const KernelKey &, const ReduceParams &r, cudaStream_t s) {      \
+    cudaError_t launch_reduce_##SUFFIX(const KernelKey &, const ForceParams &r, cudaStream_t s) {       \
         return launch_reduce<POLICY>(r, s);                                                             \
     }                                                                                                   \
     cudaError_t launch_batched_##SUFFIX(int, const BatchParams &, int, int, cudaStream_t) {             \

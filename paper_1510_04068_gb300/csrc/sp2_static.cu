@@ -175,21 +175,10 @@ extern "C" sp2_status sp2_step_static(int64_t n_j, const int32_t *id, const doub
     int32_t *part_id = reinterpret_cast<int32_t *>(part_base + static_cast<size_t>(split) * n_i * (kFields + nn) * sizeof(double));
     fp.part = part;
     fp.part_id = part_id;
-    fp.sink_major = split >= kWarpReduceMinSplit ? 1 : 0;
     const int grid = static_cast<int>(std::min<int64_t>(fp.n_items, static_cast<int64_t>(sms) * per_sm));
     if (launch_force_kernel(key, fp, grid, L.threads, L.j_tile, s) != cudaSuccess) return SP2_ERR_CUDA;
     if (split > 1) {
-        ReduceParams r{};
-        r.part = part;
-        r.part_id = part_id;
-        r.n_i = n_i;
-        r.split = static_cast<int>(split);
-        r.acc = acc;
-        r.jerk = jerk_out;
-        r.pot = pot;
-        r.nn_id = nn_id;
-        r.nn_r2 = nn_r2;
-        if (launch_reduce_kernel(key, r, s) != cudaSuccess) return SP2_ERR_CUDA;
+        if (launch_reduce_kernel(key, fp, s) != cudaSuccess) return SP2_ERR_CUDA;
     }
     mark_bad_sinks_kernel<<<static_cast<unsigned>(ceil_div(n_i, 256)), 256, 0, s>>>(i_idx, n_i, n_j, acc, jerk_out,
                                                                                     pot, nn_id, nn_r2);
