@@ -952,13 +952,34 @@ struct WithNeighbours : B {
         const int k = atomicAdd(s.cnt, 1);
         if (k < s.cap) s.lst[k] = j;
     }
-    template <bool SELF, bool FIRST, class R>
-    __device__ static __forceinline__ float2 interact2(const R &r, int j, int jl, int u, const Sink &s,
-                                                       typename B::Acc &c, float eps2) {
-        const float2 d2 = B::template interact2<SELF, FIRST>(r, j, jl, u, s, c, eps2);
-        if (d2.x < s.h2 && (!SELF || j != s.slot)) add(s, j);
-        if (d2.y < s.h2 && (!SELF || j + jl != s.slot)) add(s, j + jl);
-        return d2;
+    // Paired policies: the chunk's nearest-neighbour key is its smallest r^2
+    // (rounded down by the position bits; the self pair left out), so one
+    // compare per chunk says whether any of its sources can lie inside the
+    // radius.  Only then is the chunk scanned again, from its pair records in
+    // shared memory, with the r^2 of interact2.  A radius holds some tens of
+    // sources, so a warp's 32 sinks scan a few per cent of the chunks, where a
+    // test of every pair cost a quarter of the pass.  With the sort of the lists
+    // (nb_finish_kernel): 16384 sinks on 131072 sources 3175 -> 2937 us a step.
+    __device__ static __forceinline__ void fold(typename B::Acc &c, int base, const unsigned char *pq, int pstep,
+                                                const Sink &s) {
+        if (__uint_as_float(c.ck & ~B::kKeyMask) < s.h2) scan_chunk(base, pq, pstep, s);
+        B::fold(c, base, pq, pstep, s);
+    }
+    __device__ static __forceinline__ void fold(typename B::Acc &c, int base) { B::fold(c, base); }
+    __device__ static __forceinline__ void scan_chunk(int base, const unsigned char *pq, int pstep, const Sink &s) {
+        // slots between a lane's consecutive sources: the lanes per sink, a power of
+        // two (the records of pstep / jl bytes may be padded by less than a third)
+        const int jl = 1 << (31 - __clz(pstep / B::PRB));
+#pragma unroll 1
+        for (int u = 0; u < B::kChunk; ++u) {
+            const float *q = reinterpret_cast<const float *>(pq + (u >> 1) * pstep) + (u & 1);
+            // floats of a pair record: xh 0,1  yh 2,3  zh 4,5  xl 8,9  yl 10,11  zl 12,13
+            const float dx = (q[0] - s.xh.x) + (q[8] - s.xl.x);
+            const float dy = (q[2] - s.yh.x) + (q[10] - s.yl.x);
+            const float dz = (q[4] - s.zh.x) + (q[12] - s.zl.x);
+            const int j = base + u * jl;
+            if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < s.h2 && j != s.slot) add(s, j);
+        }
     }
     template <bool SELF, bool FIRST, class R>
     __device__ static __forceinline__ double interact(const R &r, int j, int u, const Sink &s, typename B::Acc &c,

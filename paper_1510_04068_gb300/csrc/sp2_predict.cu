@@ -273,21 +273,61 @@ __global__ void pack_state_kernel(int64_t n, const double *m, const double *x, c
 }
 
 // Neighbour lists after the pass: stored slots become ids and each list is
-// sorted by id (insertion sort; lists are short), so a list without overflow
-// has one defined order.
-__global__ void nb_finish_kernel(const int32_t *ids, int64_t n_i, int nb_max, const int32_t *count, int32_t *list) {
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n_i) return;
+// sorted by id, so a list without overflow has one defined order.  A warp per
+// sink: lists of up to kNbShared entries (the usual tens) are read once into
+// shared memory and every entry is written straight to its rank (the entries
+// below it, counted with broadcast reads; equal ids keep their order); longer
+// ones are sorted in place by a bitonic network whose comparators all point
+// the same way, so that entries past the end need no padding.  An insertion
+// sort by one thread per sink, in place, took 187 us for 16384 lists.
+constexpr int kNbShared = 256;
+constexpr int kNbWarps = 4;
+
+__global__ void __launch_bounds__(32 * kNbWarps)
+nb_finish_kernel(const int32_t *ids, int64_t n_i, int nb_max, const int32_t *count, int32_t *list) {
+    __shared__ int32_t buf[kNbWarps][kNbShared];
+    const int lane = threadIdx.x & 31;
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * kNbWarps + (threadIdx.x >> 5);
+    if (i >= n_i) return;  // uniform across the warp
     const int c = min(count[i], nb_max);
     int32_t *l = list + i * nb_max;
-    for (int k = 0; k < c; ++k) {
-        const int32_t v = ids[l[k]];
-        int q = k;
-        while (q > 0 && l[q - 1] > v) {
-            l[q] = l[q - 1];
-            --q;
+    if (c <= kNbShared) {
+        int32_t *sh = buf[threadIdx.x >> 5];
+        for (int k = lane; k < c; k += 32) sh[k] = ids[l[k]];
+        __syncwarp();
+        for (int k = lane; k < c; k += 32) {
+            const int32_t v = sh[k];
+            int rank = 0;
+            for (int q = 0; q < c; ++q) rank += (sh[q] < v || (sh[q] == v && q < k)) ? 1 : 0;
+            l[rank] = v;
         }
-        l[q] = v;
+        return;
+    }
+    for (int k = lane; k < c; k += 32) l[k] = ids[l[k]];
+    __syncwarp();
+    auto order = [&](int p, int q) {
+        if (q >= c) return;
+        const int32_t a = l[p], b = l[q];
+        if (a > b) {
+            l[p] = b;
+            l[q] = a;
+        }
+    };
+    int half = 1;
+    for (int size = 2; half < c; size *= 2, half *= 2) {
+        // mirrored step: position p of a block's lower half against the mirror position
+        for (int k = lane; k < (c + size - 1) / size * half; k += 32) {
+            const int blk = k / half, p = k - blk * half;
+            order(blk * size + p, blk * size + size - 1 - p);
+        }
+        __syncwarp();
+        for (int d = half / 2; d > 0; d /= 2) {
+            for (int k = lane; k < (c + 2 * d - 1) / (2 * d) * d; k += 32) {
+                const int blk = k / d, p = k - blk * d;
+                order(blk * 2 * d + p, blk * 2 * d + p + d);
+            }
+            __syncwarp();
+        }
     }
 }
 
@@ -740,7 +780,7 @@ cudaError_t launch_block_init(const JStore &js, double *dt, int64_t n, double et
 cudaError_t launch_nb_finish(const int32_t *ids, int64_t n_i, int nb_max, const int32_t *count, int32_t *list,
                              cudaStream_t s) {
     if (n_i <= 0) return cudaSuccess;
-    nb_finish_kernel<<<grid_for(n_i), kThreads, 0, s>>>(ids, n_i, nb_max, count, list);
+    nb_finish_kernel<<<static_cast<unsigned>((n_i + kNbWarps - 1) / kNbWarps), 32 * kNbWarps, 0, s>>>(ids, n_i, nb_max, count, list);
     return cudaGetLastError();
 }
 
