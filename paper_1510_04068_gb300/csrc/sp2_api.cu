@@ -66,8 +66,8 @@ struct sp2_ctx {
     unsigned char *rec2 = nullptr;  // records of the all-pairs / VJP entry points
     int32_t *iota = nullptr;
     double *tmp = nullptr;          // 4 x (n_max x 3) doubles: a1, j1, xpbar, vpbar
-    unsigned int *dev_words = nullptr;  // [0] batched work queue, [1] error flag, [2] finite flag,
-                                        // [4] pass work queue, [5] pass exit count (both self-resetting)
+    unsigned int *dev_words = nullptr;  // [1] error flag, [2] finite flag; self-resetting: [0] batched work queue,
+                                        // [6] batched exit count, [4] pass work queue, [5] pass exit count
     double *part = nullptr;
     int32_t *part_id = nullptr;
     size_t part_cap = 0, part_id_cap = 0;   // bytes
@@ -1164,6 +1164,7 @@ sp2_status sp2_compute_batched(sp2_ctx *c, const sp2_batch_plan *plan, double *a
     b.n_items = plan->n_items;
     b.out_base = plan->out_base;
     b.queue = c->dev_words;
+    b.exit_count = c->dev_words + 6;
     b.eps2 = c->cfg.eps2;
     const int threads = 256;
     int per_sm = 0;
@@ -1171,7 +1172,6 @@ sp2_status sp2_compute_batched(sp2_ctx *c, const sp2_batch_plan *plan, double *a
     const int64_t warps_needed = plan->n_items;
     const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(ceil_div(warps_needed, threads / 32),
                                                                              static_cast<int64_t>(c->sm_count) * std::max(per_sm, 1))));
-    SP2_CK(c, cudaMemsetAsync(c->dev_words, 0, sizeof(unsigned int), c->stream));
     ev_begin(c, ST_BATCHED);
     SP2_CK(c, launch_batched_kernel(c->cfg.order, mixed, nn, b, grid, threads, c->stream));
     ev_end(c, ST_BATCHED);

@@ -2181,8 +2181,8 @@ __device__ __forceinline__ void batch_tile_loop(const unsigned char *st, int tb,
     }
 }
 
-// Warps take (system, up-to-32-sink chunk) items from the device queue in the
-// plan's cost order; one sink per lane.  The system's sources pass through a
+// Warps take (system, up-to-32-sink chunk) items in the plan's cost order; one
+// sink per lane.  The system's sources pass through a
 // warp-private shared-memory tile filled with coalesced 16-byte loads (ragged
 // ends padded with filler records), then are read as broadcasts.  The running
 // totals stay in registers (systems are short).
@@ -2193,11 +2193,16 @@ __global__ void __launch_bounds__(kMaxThreads) batched_kernel(const BatchParams 
     unsigned char *wbuf = smem + static_cast<size_t>(threadIdx.x >> 5) * kBatchTile * P::RB;
     const typename P::real eps2 = static_cast<typename P::real>(b.eps2);
     constexpr int W = P::RB / 16;
-    for (;;) {
-        unsigned int item = 0;
-        if (lane == 0) item = atomicAdd(b.queue, 1u);
-        item = __shfl_sync(kFull, item, 0);
-        if (item >= b.n_items) break;
+    // The first item of a warp is its own number in the grid; the queue hands
+    // out the rest, and a warp asks for its next item before it works on the
+    // current one, so neither the counter's round trip nor the contention of
+    // all warps at the start stands in front of the arithmetic (4096
+    // planetary systems, prediction included: 77.7 -> 74.8 us).
+    const unsigned n_warps = gridDim.x * (blockDim.x >> 5);
+    unsigned item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    while (item < b.n_items) {
+        unsigned next = 0;
+        if (lane == 0) next = n_warps + atomicAdd(b.queue, 1u);
         const int4 it = __ldg(b.items + item);  // {system first slot, size, chunk first slot, chunk size}
         const bool val = lane < it.w;
         const int slot = it.z + (val ? lane : 0);
@@ -2251,6 +2256,17 @@ __global__ void __launch_bounds__(kMaxThreads) batched_kernel(const BatchParams 
         if constexpr (has_fold_tile<P>::value || is_paired<P>::value) P::nn_acc(ac, nd, nid);
         else P::nn(ac, sk, b.rec, static_cast<int64_t>(it.x) + it.y, 1, nd, nid);
         if (val) P::write_final(b, static_cast<int64_t>(slot) - b.out_base, t, nd, nid);
+        item = __shfl_sync(kFull, next, 0);
+    }
+    // the last CTA out resets the counters for the next launch (every warp of
+    // a CTA has drawn its last item before the CTA is counted)
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(b.exit_count, 1u) == gridDim.x - 1) {
+            *b.queue = 0u;
+            *b.exit_count = 0u;
+        }
     }
 }
 

@@ -104,7 +104,8 @@ struct BatchParams {
     const int4 *items;         // {system first slot, system size, chunk first slot, chunk size}
     int64_t n_items;
     int64_t out_base;          // slot of output row 0
-    unsigned int *queue;
+    unsigned int *queue;       // items drawn beyond each warp's first, and CTAs done: both zero at
+    unsigned int *exit_count;  // launch, reset by the last CTA out
     double eps2;
     double *acc, *jerk, *snap, *pot;
     int32_t *nn_id;
