@@ -1335,7 +1335,10 @@ static sp2_status block_run_impl(sp2_ctx *c, double t_end, double eta, double et
     BlockDev h{};
     h.min_active = 0xffffffffu;
     h.t_last = -1.0;
+    for (unsigned long long &q : h.t1bits) q = ~0ull;
     SP2_CK(c, cudaMemcpyAsync(c->blk_dev, &h, sizeof h, cudaMemcpyHostToDevice, c->stream));
+    SP2_CK(c, launch_block_first(c->js.t, c->blk_dt, n, c->blk_dev, c->stream));
+    c->launches += 1;
     // The active count is only known on the device: the pass kernel derives
     // its sinks per CTA and source split from it.  The host fixes the CTA
     // (256 threads, one sink per thread), the tile (256 sources, room for 32
@@ -1365,26 +1368,22 @@ static sp2_status block_run_impl(sp2_ctx *c, double t_end, double eta, double et
     // the device and every later kernel of the batch does nothing.  The first
     // batch is launched directly (it sizes the pass buffers); the rest replay
     // one captured batch as a CUDA graph.
-    constexpr int kBatch = 32;
+    constexpr int kBatch = 32;  // a multiple of 4, the slots of the run state
     auto enqueue = [&]() -> sp2_status {
         for (int k = 0; k < kBatch; ++k) {
-            ev_begin(c, ST_OTHER);
-            SP2_CK(c, launch_block_begin(c->blk_dev, c->js.t, c->blk_dt, n, t_end, c->blk_active, c->stream));
-            ev_end(c, ST_OTHER);
+            const BlockStep b{c->blk_dev, c->js.t, c->blk_dt, c->blk_active, t_end, k & 3};
             ev_begin(c, ST_PREDICT);
-            SP2_CK(c, launch_predict(order, mixed, jp, n, 0.0, c->rec, c->stream, c->blk_dev));
+            SP2_CK(c, launch_block_predict(order, mixed, jp, n, c->rec, b, c->stream));
             ev_end(c, ST_PREDICT);
             SP2_CKS(run_pass(c, K_FORCE, order, mixed, 0, c->rec, c->rb, n, c->blk_active, n, 0, n, o, &L, ST_FORCE,
-                             nullptr, false, &c->blk_dev->count));
+                             nullptr, false, &c->blk_dev->count[b.slot]));
             ev_begin(c, ST_OTHER);
             if (order == 6)
-                SP2_CK(c, launch_block_correct6_dev(jc, c->blk_dt, c->blk_active, n, c->blk_dev, a1, j1, s1, eta,
-                                                    eta6, dt_max, c->stream));
+                SP2_CK(c, launch_block_correct6_dev(jc, b, n, a1, j1, s1, eta, eta6, dt_max, c->stream));
             else
-                SP2_CK(c, launch_block_correct_dev(jc, c->blk_dt, c->blk_active, n, c->blk_dev, a1, j1, eta, dt_max,
-                                                   c->stream));
+                SP2_CK(c, launch_block_correct_dev(jc, b, n, a1, j1, eta, dt_max, c->stream));
             ev_end(c, ST_OTHER);
-            c->launches += 5;  // run_pass counts the force kernel
+            c->launches += 2;  // run_pass counts the force kernel
         }
         return SP2_OK;
     };

@@ -2090,6 +2090,9 @@ __device__ __forceinline__ void device_shape(ForceParams &q) {
     q.n_items = n_iblk * q.split;
     q.sinks_per_cta = spc;
     q.jl = jl;
+    // every item its own CTA: no draw from the work queue (two round trips to
+    // its counter per CTA) where the items fit the grid
+    q.static_items = q.n_items <= static_cast<int64_t>(gridDim.x) ? 1 : 0;
 }
 
 // Resident CTAs of kMaxThreads that a kernel's register budget must allow

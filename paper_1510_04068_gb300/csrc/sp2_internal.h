@@ -172,20 +172,29 @@ cudaError_t launch_scatter_j(const JStore &dst, const int32_t *slots, int64_t n,
                              const double *t, cudaStream_t s);
 // State of a device-driven block time-step run (one per context).
 struct BlockDev {
-    unsigned long long t1bits;  // order-preserving key of the current block time
-    unsigned int count;         // active particles of the current block (0: none / stopped)
+    // block b uses slot b % 4 (see block_select)
+    unsigned long long t1bits[4];  // order-preserving key of the block's time
+    unsigned int count[4];         // active particles of the block (0: none / stopped)
     unsigned int stop;          // set once the next block time passes t_end (or on underflow)
     unsigned int underflow;     // a new step fell to the 2^-50 floor: the run stops there
     unsigned long long steps, active_sum;
     unsigned int max_active, min_active;
     double t_last;              // time of the last block taken
 };
+// One block of a run: the state, its slot and the particles' times and steps.
+struct BlockStep {
+    BlockDev *bd;
+    const double *t;
+    double *dt;
+    int32_t *active;  // active slots of the current block
+    double t_end;
+    int slot;
+};
 
 // Mixed records come from js.dsc when it is set (double-single arithmetic),
-// from the FP64 arrays otherwise.  t_dev: if set, the time is read on the
-// device from a BlockDev (the launch does nothing when its count is zero)
+// from the FP64 arrays otherwise.
 cudaError_t launch_predict(int order, int mixed, const JStore &js, int64_t n, double t,
-                           unsigned char *rec, cudaStream_t s, const BlockDev *t_dev = nullptr);
+                           unsigned char *rec, cudaStream_t s);
 // Refresh js.dsc for slots [first, first + n) from the FP64 store.
 cudaError_t launch_dscache(int order, const JStore &js, int64_t first, int64_t n, cudaStream_t s);
 // (m, x, v) -> order-4 records with no prediction (all-pairs entry points)
@@ -199,19 +208,20 @@ cudaError_t launch_iota(int32_t *dst, int64_t n, cudaStream_t s);
 // Block time-steps (Hermite-4 with individual power-of-two steps).
 cudaError_t launch_block_init(const JStore &js, double *dt, int64_t n, double eta_s, double dt_max, double t0,
                               cudaStream_t s);
-// bd->t1bits = key of t1 = min(t + dt); active[0 .. bd->count) = slots with
-// t + dt == t1, or bd->stop set (count 0) once t1 > t_end
-cudaError_t launch_block_begin(BlockDev *bd, const double *t, const double *dt, int64_t n, double t_end,
-                               int32_t *active, cudaStream_t s);
-// Hermite-4 corrector and new step of the active slots of the current block
-cudaError_t launch_block_correct_dev(const JStore &js, double *dt, const int32_t *active, int64_t n_max,
-                                     BlockDev *bd, const double *a1, const double *j1, double eta, double dt_max,
-                                     cudaStream_t s);
+// the first block time of a run: slot 0 of bd->t1bits (all ones before) = key of min(t + dt)
+cudaError_t launch_block_first(const double *t, const double *dt, int64_t n, BlockDev *bd, cudaStream_t s);
+// selects the active slots of block b (count 0 and bd->stop set once its time
+// is past t_end) and predicts all particles to its time
+cudaError_t launch_block_predict(int order, int mixed, const JStore &js, int64_t n, unsigned char *rec,
+                                 const BlockStep &b, cudaStream_t s);
+// Hermite-4 corrector and new step of the active slots of block b
+cudaError_t launch_block_correct_dev(const JStore &js, const BlockStep &b, int64_t n_max, const double *a1,
+                                     const double *j1, double eta, double dt_max, cudaStream_t s);
 // 6th-order form: s1 the snaps, js.cr the crackles (updated), the averaged
 // criterion with eta4 and eta6
-cudaError_t launch_block_correct6_dev(const JStore &js, double *dt, const int32_t *active, int64_t n_max,
-                                      BlockDev *bd, const double *a1, const double *j1, const double *s1,
-                                      double eta4, double eta6, double dt_max, cudaStream_t s);
+cudaError_t launch_block_correct6_dev(const JStore &js, const BlockStep &b, int64_t n_max, const double *a1,
+                                      const double *j1, const double *s1, double eta4, double eta6, double dt_max,
+                                      cudaStream_t s);
 cudaError_t launch_nb_finish(const int32_t *ids, int64_t n_i, int nb_max, const int32_t *count, int32_t *list,
                              cudaStream_t s);
 cudaError_t launch_h4_predict_pack(int mixed, int64_t n, double dt, const double *m,

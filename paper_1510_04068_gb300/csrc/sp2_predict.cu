@@ -148,18 +148,56 @@ __device__ __forceinline__ double key_time(unsigned long long k) {
     return __longlong_as_double(static_cast<long long>(b));
 }
 
+// minimum over a warp's lanes into *dst (all ones: nothing to add)
+__device__ __forceinline__ void warp_min_to(unsigned long long *dst, unsigned long long v) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, off));
+    if ((threadIdx.x & 31) == 0 && v != ~0ull) atomicMin(dst, v);
+}
+
+// Block time-steps: the start of block b, run by every thread of the
+// prediction (slot j; threads past n take part in the warp's minimum).  The
+// block time is in slot b % 4 of the run state; particles due then are
+// appended to the active list, and the next due time of all others goes into
+// slot (b + 1) % 4, to which the corrector adds the active particles' new
+// times: no pass over the particles is spent on finding the next block time.
+// The slots of the blocks after that are reset on the way (nothing reads or
+// writes them during block b).  Returns false when the run has stopped or the
+// block time is past t_end (which stops it: the counts stay 0 and every later
+// kernel does nothing).
+__device__ __forceinline__ bool block_select(const BlockStep &b, int64_t j, int64_t n, double *t1) {
+    BlockDev *bd = b.bd;
+    if (j == 0) bd->count[(b.slot + 1) & 3] = 0u;  // (also once stopped: every count must be 0 then)
+    if (bd->stop) return false;
+    *t1 = key_time(bd->t1bits[b.slot]);
+    if (!(*t1 <= b.t_end)) {
+        if (j == 0) bd->stop = 1u;
+        return false;
+    }
+    if (j == 0) bd->t1bits[(b.slot + 2) & 3] = ~0ull;
+    unsigned long long next = ~0ull;
+    if (j < n) {
+        const double due = b.t[j] + b.dt[j];
+        if (due == *t1) b.active[atomicAdd(&bd->count[b.slot], 1u)] = static_cast<int32_t>(j);
+        else next = time_key(due);
+    }
+    warp_min_to(&bd->t1bits[(b.slot + 1) & 3], next);
+    return true;
+}
+
 // Mixed-precision predictor on the double-single cache (predict_ds_record).
-template <int ORDER>
+// BLOCK: to the time of the current block, whose active set it selects.
+template <int ORDER, bool BLOCK>
 __global__ void predict_ds_kernel(const float4 *dsc, int64_t n, float t_hi, float t_lo, unsigned char *rec,
-                                  const BlockDev *bd) {
+                                  const BlockStep b) {
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    if (bd) {  // time of the current block, chosen on the device
-        if (bd->count == 0) return;
-        const double t = key_time(bd->t1bits);
+    if constexpr (BLOCK) {
+        double t;
+        if (!block_select(b, j, n, &t)) return;
         t_hi = __double2float_rn(t);
         t_lo = __double2float_rn(t - static_cast<double>(t_hi));
     }
+    if (j >= n) return;
     float4 o[4];
     predict_ds_record<ORDER>(dsc, j, t_hi, t_lo, o);
     float4 *dst = reinterpret_cast<float4 *>(rec + j * (ORDER == 6 ? 64 : 48));
@@ -205,14 +243,13 @@ scatter_kernel(JStore d, const int32_t *slots, int64_t n, int64_t n_loaded, unsi
     if (d.dsc) write_dscache_vec(d, s, c, xx, vv, aa, jj, ss);
 }
 
-template <int ORDER, bool MIXED>
-__global__ void predict_kernel(JStore js, int64_t n, double t, unsigned char *rec, const BlockDev *bd) {
+template <int ORDER, bool MIXED, bool BLOCK>
+__global__ void predict_kernel(JStore js, int64_t n, double t, unsigned char *rec, const BlockStep b) {
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    if (bd) {
-        if (bd->count == 0) return;
-        t = key_time(bd->t1bits);
+    if constexpr (BLOCK) {
+        if (!block_select(b, j, n, &t)) return;
     }
+    if (j >= n) return;
     const double c2 = 0.5, c3 = 1.0 / 6.0, c4 = 1.0 / 24.0;
     const double dt = dadd(t, -js.t[j]);
     const double dt2 = dmul(dt, dt);
@@ -437,50 +474,35 @@ __global__ void pack_sinks_kernel(int64_t n, const double *x, const double *v, c
 // ---- the same block time-steps driven from the device: the block time,
 // the active count and a stop flag live in a BlockDev, so the host can queue
 // many blocks without reading anything back.
-__global__ void block_begin_kernel(BlockDev *bd) {
-    bd->count = 0u;
-    if (!bd->stop) bd->t1bits = ~0ull;
-}
-
-__global__ void block_next_dev_kernel(const double *t, const double *dt, int64_t n, BlockDev *bd) {
-    if (bd->stop) return;
+// The first block time of a run: the smallest t + dt, into slot 0.
+__global__ void block_first_kernel(const double *t, const double *dt, int64_t n, BlockDev *bd) {
     const int64_t s = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    unsigned long long v = ~0ull;
-    if (s < n) v = static_cast<unsigned long long>(time_key(t[s] + dt[s]));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, off));
-    if ((threadIdx.x & 31) == 0 && v != ~0ull) atomicMin(&bd->t1bits, v);
+    warp_min_to(&bd->t1bits[0], s < n ? time_key(t[s] + dt[s]) : ~0ull);
 }
 
-// active set of the block, unless the block time has passed t_end (then the
-// run stops: count stays 0 and every later kernel of the run does nothing)
-__global__ void block_active_dev_kernel(const double *t, const double *dt, int64_t n, double t_end, BlockDev *bd,
-                                        int32_t *active) {
-    if (bd->stop) return;
-    const double t1 = key_time(bd->t1bits);
-    if (!(t1 <= t_end)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) bd->stop = 1u;
-        return;
-    }
-    const int64_t s = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (s < n && t[s] + dt[s] == t1) active[atomicAdd(&bd->count, 1u)] = static_cast<int32_t>(s);
+// The run's statistics (first thread of a corrector).
+__device__ __forceinline__ void count_block(BlockDev *bd, unsigned int n_act, double t1) {
+    bd->steps += 1;
+    bd->active_sum += n_act;
+    bd->max_active = max(bd->max_active, n_act);
+    bd->min_active = min(bd->min_active, n_act);
+    bd->t_last = t1;
 }
 
-__global__ void block_correct_dev_kernel(JStore js, double *dt, const int32_t *active, BlockDev *bd, const double *a1,
-                                         const double *j1, double eta, double dt_max) {
+__global__ void block_correct_dev_kernel(JStore js, const BlockStep b, const double *a1, const double *j1, double eta,
+                                         double dt_max) {
     const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    const unsigned int n_act = bd->count;
-    const double t1 = key_time(bd->t1bits);
-    if (k == 0 && n_act > 0) {
-        bd->steps += 1;
-        bd->active_sum += n_act;
-        bd->max_active = max(bd->max_active, n_act);
-        bd->min_active = min(bd->min_active, n_act);
-        bd->t_last = t1;
+    const unsigned int n_act = b.bd->count[b.slot];
+    const double t1 = key_time(b.bd->t1bits[b.slot]);
+    if (k == 0 && n_act > 0) count_block(b.bd, n_act, t1);
+    unsigned long long next = ~0ull;
+    if (k < n_act) {
+        const int64_t s = b.active[k];
+        correct_one(js, b.dt, s, k, t1, a1, j1, eta, dt_max);
+        check_underflow(b.dt, s, b.bd);
+        next = time_key(t1 + b.dt[s]);
     }
-    if (k >= n_act) return;
-    correct_one(js, dt, active[k], k, t1, a1, j1, eta, dt_max);
-    check_underflow(dt, active[k], bd);
+    warp_min_to(&b.bd->t1bits[(b.slot + 1) & 3], next);
 }
 
 // 6th-order Hermite corrector (Nitadori & Makino 2008) for slot s, position k
@@ -538,22 +560,20 @@ __device__ __forceinline__ void correct6_one(const JStore &js, double *dt, int64
     if (js.dsc) write_dscache(js, s);
 }
 
-__global__ void block_correct6_dev_kernel(JStore js, double *dt, const int32_t *active, BlockDev *bd,
-                                          const double *a1, const double *j1, const double *s1, double eta4,
-                                          double eta6, double dt_max) {
+__global__ void block_correct6_dev_kernel(JStore js, const BlockStep b, const double *a1, const double *j1,
+                                          const double *s1, double eta4, double eta6, double dt_max) {
     const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    const unsigned int n_act = bd->count;
-    const double t1 = key_time(bd->t1bits);
-    if (k == 0 && n_act > 0) {
-        bd->steps += 1;
-        bd->active_sum += n_act;
-        bd->max_active = max(bd->max_active, n_act);
-        bd->min_active = min(bd->min_active, n_act);
-        bd->t_last = t1;
+    const unsigned int n_act = b.bd->count[b.slot];
+    const double t1 = key_time(b.bd->t1bits[b.slot]);
+    if (k == 0 && n_act > 0) count_block(b.bd, n_act, t1);
+    unsigned long long next = ~0ull;
+    if (k < n_act) {
+        const int64_t s = b.active[k];
+        correct6_one(js, b.dt, s, k, t1, a1, j1, s1, eta4, eta6, dt_max);
+        check_underflow(b.dt, s, b.bd);
+        next = time_key(t1 + b.dt[s]);
     }
-    if (k >= n_act) return;
-    correct6_one(js, dt, active[k], k, t1, a1, j1, s1, eta4, eta6, dt_max);
-    check_underflow(dt, active[k], bd);
+    warp_min_to(&b.bd->t1bits[(b.slot + 1) & 3], next);
 }
 
 __global__ void iota_kernel(int32_t *dst, int64_t n) {
@@ -690,31 +710,45 @@ cudaError_t launch_dscache(int order, const JStore &js, int64_t first, int64_t n
     return cudaGetLastError();
 }
 
-cudaError_t launch_predict(int order, int mixed, const JStore &js, int64_t n, double t, unsigned char *rec,
-                           cudaStream_t s, const BlockDev *bd) {
-    if (n <= 0) return cudaSuccess;
+namespace {
+template <bool BLOCK>
+cudaError_t launch_predict_form(int order, int mixed, const JStore &js, int64_t n, double t, unsigned char *rec,
+                                cudaStream_t s, const BlockStep &b) {
     const unsigned g = grid_for(n);
     if (mixed && js.dsc) {
         const float th = static_cast<float>(t);
         const float tl = static_cast<float>(t - static_cast<double>(th));
-        if (order == 6) predict_ds_kernel<6><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, bd);
-        else if (order == 2) predict_ds_kernel<2><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, bd);
-        else predict_ds_kernel<4><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, bd);
+        if (order == 6) predict_ds_kernel<6, BLOCK><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, b);
+        else if (order == 2) predict_ds_kernel<2, BLOCK><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, b);
+        else predict_ds_kernel<4, BLOCK><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, b);
         return cudaGetLastError();
     }
     // the FP64 predictor is FP64-bound: 64-thread CTAs spread it over the SMs
     const unsigned g64 = static_cast<unsigned>((n + 63) / 64);
     if (order == 6) {
-        if (mixed) predict_kernel<6, true><<<g64, 64, 0, s>>>(js, n, t, rec, bd);
-        else predict_kernel<6, false><<<g64, 64, 0, s>>>(js, n, t, rec, bd);
+        if (mixed) predict_kernel<6, true, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
+        else predict_kernel<6, false, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
     } else if (order == 2) {
-        if (mixed) predict_kernel<2, true><<<g64, 64, 0, s>>>(js, n, t, rec, bd);
-        else predict_kernel<2, false><<<g64, 64, 0, s>>>(js, n, t, rec, bd);
+        if (mixed) predict_kernel<2, true, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
+        else predict_kernel<2, false, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
     } else {
-        if (mixed) predict_kernel<4, true><<<g64, 64, 0, s>>>(js, n, t, rec, bd);
-        else predict_kernel<4, false><<<g64, 64, 0, s>>>(js, n, t, rec, bd);
+        if (mixed) predict_kernel<4, true, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
+        else predict_kernel<4, false, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
     }
     return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_predict(int order, int mixed, const JStore &js, int64_t n, double t, unsigned char *rec,
+                           cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    return launch_predict_form<false>(order, mixed, js, n, t, rec, s, BlockStep{});
+}
+
+cudaError_t launch_block_predict(int order, int mixed, const JStore &js, int64_t n, unsigned char *rec,
+                                 const BlockStep &b, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    return launch_predict_form<true>(order, mixed, js, n, 0.0, rec, s, b);
 }
 
 cudaError_t launch_pack_state(int mixed, int64_t n, const double *m, const double *x, const double *v,
@@ -745,28 +779,24 @@ cudaError_t launch_iota(int32_t *dst, int64_t n, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_block_begin(BlockDev *bd, const double *t, const double *dt, int64_t n, double t_end,
-                               int32_t *active, cudaStream_t s) {
-    block_begin_kernel<<<1, 1, 0, s>>>(bd);
-    block_next_dev_kernel<<<grid_for(n), kThreads, 0, s>>>(t, dt, n, bd);
-    block_active_dev_kernel<<<grid_for(n), kThreads, 0, s>>>(t, dt, n, t_end, bd, active);
+cudaError_t launch_block_first(const double *t, const double *dt, int64_t n, BlockDev *bd, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    block_first_kernel<<<grid_for(n), kThreads, 0, s>>>(t, dt, n, bd);
     return cudaGetLastError();
 }
 
-cudaError_t launch_block_correct_dev(const JStore &js, double *dt, const int32_t *active, int64_t n_max,
-                                     BlockDev *bd, const double *a1, const double *j1, double eta, double dt_max,
-                                     cudaStream_t s) {
+cudaError_t launch_block_correct_dev(const JStore &js, const BlockStep &b, int64_t n_max, const double *a1,
+                                     const double *j1, double eta, double dt_max, cudaStream_t s) {
     if (n_max <= 0) return cudaSuccess;
-    block_correct_dev_kernel<<<grid_for_warps(n_max), kWarpCta, 0, s>>>(js, dt, active, bd, a1, j1, eta, dt_max);
+    block_correct_dev_kernel<<<grid_for_warps(n_max), kWarpCta, 0, s>>>(js, b, a1, j1, eta, dt_max);
     return cudaGetLastError();
 }
 
-cudaError_t launch_block_correct6_dev(const JStore &js, double *dt, const int32_t *active, int64_t n_max,
-                                      BlockDev *bd, const double *a1, const double *j1, const double *s1,
-                                      double eta4, double eta6, double dt_max, cudaStream_t s) {
+cudaError_t launch_block_correct6_dev(const JStore &js, const BlockStep &b, int64_t n_max, const double *a1,
+                                      const double *j1, const double *s1, double eta4, double eta6, double dt_max,
+                                      cudaStream_t s) {
     if (n_max <= 0) return cudaSuccess;
-    block_correct6_dev_kernel<<<grid_for_warps(n_max), kWarpCta, 0, s>>>(js, dt, active, bd, a1, j1, s1, eta4, eta6,
-                                                                       dt_max);
+    block_correct6_dev_kernel<<<grid_for_warps(n_max), kWarpCta, 0, s>>>(js, b, a1, j1, s1, eta4, eta6, dt_max);
     return cudaGetLastError();
 }
 
