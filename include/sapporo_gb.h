@@ -265,13 +265,11 @@ sp2_status sp2_get_j(sp2_ctx *ctx, int64_t first, int64_t n, double *x, double *
  *   its own t_i <= t_end (all at t_end when t_end is a multiple of dt_max).
  *   Statistics go to *stats (may be NULL).
  *   Execution: the block time, the active count and a stop flag stay on the
- *   device; blocks are queued 32 at a time (the first 32 as plain launches,
- *   the rest by replaying one captured CUDA graph of 32 blocks) and the host
- *   reads the state once per 32 blocks.  A block past t_end makes the rest of
- *   its batch do nothing.  The force pass takes its shape (lanes per sink,
- *   source split) from the active count on the device.  Runs on the context's
- *   stream and returns after synchronising it; a stream that cannot be
- *   captured gets plain launches throughout.
+ *   device; blocks are queued 8 at a time, three launches each, and the host
+ *   reads the state of 8 blocks while the next 8 run.  A block past t_end makes
+ *   the queued ones after it do nothing.  The force pass takes its shape (lanes
+ *   per sink, source split) from the active count on the device.  Runs on the
+ *   context's stream and returns after synchronising it.
  * sp2_block_run_h6: the same loop with the 6th-order Hermite scheme
  *   (Nitadori & Makino 2008; Sec. 3.7 runs it): the predictor carries each
  *   particle's crackle from its last correction (x to dt^5, v to dt^4, a to

@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "sp2_ds.cuh"
 #include "sp2_internal.h"
 
@@ -29,6 +31,7 @@ inline unsigned grid_for(int64_t n) { return static_cast<unsigned>((n + kThreads
 // FP64-heavy per-particle kernels over a few hundred active particles: one
 // warp per CTA spreads them over the SMs (an SM retires 2 FP64 FMAs a clock)
 constexpr int kWarpCta = 32;
+constexpr unsigned kCorrectMaxCtas = 2048;
 inline unsigned grid_for_warps(int64_t n) { return static_cast<unsigned>((n + kWarpCta - 1) / kWarpCta); }
 
 __device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
@@ -414,41 +417,64 @@ __global__ void block_init_kernel(JStore js, double *dt, int64_t n, double eta_s
 
 // Hermite-4 corrector and the next step for the active particles (a1, j1 at
 // the predicted state, position k of the active list); the double-single
-// cache follows the store.
-__device__ __forceinline__ void correct_one(const JStore &js, double *dt, int64_t s, int64_t k, double t1,
-                                            const double *a1, const double *j1, double eta, double dt_max) {
-    const double h = t1 - js.t[s];
+// cache follows the store.  Four lanes take a particle (FP64 runs at 2 lanes
+// a clock per SM, so a few hundred particles are spread over as many lanes as
+// there are): lanes c = 0..2 correct component c and lane q forms the norm
+// of the q-th of the vectors (a, j, a2, a3); every lane then has all four norms
+// and the same new step, which it returns.  Whole groups of four take part.
+// (One thread per particle took 15 us for a few hundred particles under ncu:
+// one dependent chain of some 250 FP64 operations and seven memory round trips.)
+__device__ __forceinline__ double group_get(double v, int src) { return __shfl_sync(0xffffffffu, v, src, 4); }
+
+__device__ __forceinline__ double correct_one(const JStore &js, double *dt, int64_t s, int64_t k, int c, bool valid,
+                                              double t1, const double *a1, const double *j1, double eta,
+                                              double dt_max) {
+    const bool vec = valid && c < 3, scal = valid && c == 3;
+    const int64_t q = 3 * s + c, p = 3 * k + c;
+    const double t0 = valid ? js.t[s] : 0.0;
+    const double x0 = vec ? js.x[q] : 0.0, v0 = vec ? js.v[q] : 0.0;
+    const double a0 = vec ? js.a[q] : 0.0, j0 = vec ? js.jk[q] : 0.0;
+    const double aa = vec ? a1[p] : 0.0, jj = vec ? j1[p] : 0.0;
+    const double m = scal ? js.m[s] : 0.0;
+    const int32_t id = scal ? js.id[s] : 0;
+    const double h = t1 - t0;
     const double h2 = h * h;
-    double a2[3], a3[3], an[3], jn[3];
-    for (int c = 0; c < 3; ++c) {
-        const int64_t q = 3 * s + c;
-        const double x0 = js.x[q], v0 = js.v[q], a0 = js.a[q], j0 = js.jk[q];
-        const double aa = a1[3 * k + c], jj = j1[3 * k + c];
-        const double v1 = v0 + (a0 + aa) * (h / 2) + (j0 - jj) * (h2 / 12);
-        const double x1 = x0 + (v0 + v1) * (h / 2) + (a0 - aa) * (h2 / 12);
-        const double a2_0 = (-6.0 * (a0 - aa) - h * (4.0 * j0 + 2.0 * jj)) / h2;
-        a3[c] = (12.0 * (a0 - aa) + 6.0 * h * (j0 + jj)) / (h2 * h);
-        a2[c] = a2_0 + h * a3[c];
-        an[c] = aa;
-        jn[c] = jj;
+    const double v1 = v0 + (a0 + aa) * (h / 2) + (j0 - jj) * (h2 / 12);
+    const double x1 = x0 + (v0 + v1) * (h / 2) + (a0 - aa) * (h2 / 12);
+    const double a2_0 = (-6.0 * (a0 - aa) - h * (4.0 * j0 + 2.0 * jj)) / h2;
+    const double a3 = (12.0 * (a0 - aa) + 6.0 * h * (j0 + jj)) / (h2 * h);
+    const double a2 = a2_0 + h * a3;
+    double w[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const double g0 = group_get(aa, e), g1 = group_get(jj, e), g2 = group_get(a2, e), g3 = group_get(a3, e);
+        w[e] = (c == 0) ? g0 : (c == 1) ? g1 : (c == 2) ? g2 : g3;
+    }
+    const double mine = norm3(w);
+    const double A = group_get(mine, 0), J = group_get(mine, 1), A2 = group_get(mine, 2), A3 = group_get(mine, 3);
+    const double den = J * A3 + A2 * A2;
+    const double want = (den > 0.0) ? sqrt(eta * (A * A2 + J * J) / den) : dt_max;
+    const double dn = valid ? quantise_dt(want, fmin(2.0 * h, dt_max), t1) : 0.0;
+    if (vec) {
         js.x[q] = x1;
         js.v[q] = v1;
         js.a[q] = aa;
         js.jk[q] = jj;
+        if (js.dsc) write_dscache_vec(js, s, c, x1, v1, aa, jj, 0.0);
     }
-    js.t[s] = t1;
-    const double A = norm3(an), J = norm3(jn), A2 = norm3(a2), A3 = norm3(a3);
-    const double den = J * A3 + A2 * A2;
-    const double want = (den > 0.0) ? sqrt(eta * (A * A2 + J * J) / den) : dt_max;
-    dt[s] = quantise_dt(want, fmin(2.0 * h, dt_max), t1);
-    if (js.dsc) write_dscache(js, s);
+    if (scal) {
+        js.t[s] = t1;
+        dt[s] = dn;
+        if (js.dsc) write_dscache_scalars(js, s, m, t1, id);
+    }
+    return dn;
 }
 
 // A step at the 2^-50 floor means the criterion has collapsed (Sec. 3.7 notes
 // that noisy jerk and snap can drive the step to zero): the run stops after
 // this block and the host reports it.
-__device__ __forceinline__ void check_underflow(const double *dt, int64_t s, BlockDev *bd) {
-    if (dt[s] <= kBlockDtMin) {
+__device__ __forceinline__ void check_underflow(double dt, BlockDev *bd) {
+    if (dt <= kBlockDtMin) {
         bd->underflow = 1u;
         bd->stop = 1u;
     }
@@ -489,18 +515,23 @@ __device__ __forceinline__ void count_block(BlockDev *bd, unsigned int n_act, do
     bd->t_last = t1;
 }
 
-__global__ void block_correct_dev_kernel(JStore js, const BlockStep b, const double *a1, const double *j1, double eta,
-                                         double dt_max) {
-    const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kWarpCta)
+block_correct_dev_kernel(JStore js, const BlockStep b, const double *a1, const double *j1, double eta, double dt_max) {
+    constexpr int kPer = kWarpCta / kLanesPerParticle;  // particles of a CTA (one warp) at a time
     const unsigned int n_act = b.bd->count[b.slot];
     const double t1 = key_time(b.bd->t1bits[b.slot]);
-    if (k == 0 && n_act > 0) count_block(b.bd, n_act, t1);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && n_act > 0) count_block(b.bd, n_act, t1);
+    const int c = threadIdx.x % kLanesPerParticle;
     unsigned long long next = ~0ull;
-    if (k < n_act) {
-        const int64_t s = b.active[k];
-        correct_one(js, b.dt, s, k, t1, a1, j1, eta, dt_max);
-        check_underflow(b.dt, s, b.bd);
-        next = time_key(t1 + b.dt[s]);
+    for (unsigned int k0 = blockIdx.x * kPer; k0 < n_act; k0 += gridDim.x * kPer) {  // uniform across the warp
+        const unsigned int k = k0 + threadIdx.x / kLanesPerParticle;
+        const bool valid = k < n_act;
+        const int64_t s = valid ? b.active[k] : 0;
+        const double dn = correct_one(js, b.dt, s, k, c, valid, t1, a1, j1, eta, dt_max);
+        if (valid) {
+            if (c == 3) check_underflow(dn, b.bd);
+            next = min(next, time_key(t1 + dn));
+        }
     }
     warp_min_to(&b.bd->t1bits[(b.slot + 1) & 3], next);
 }
@@ -570,7 +601,7 @@ __global__ void block_correct6_dev_kernel(JStore js, const BlockStep b, const do
     if (k < n_act) {
         const int64_t s = b.active[k];
         correct6_one(js, b.dt, s, k, t1, a1, j1, s1, eta4, eta6, dt_max);
-        check_underflow(b.dt, s, b.bd);
+        check_underflow(b.dt[s], b.bd);
         next = time_key(t1 + b.dt[s]);
     }
     warp_min_to(&b.bd->t1bits[(b.slot + 1) & 3], next);
@@ -788,7 +819,9 @@ cudaError_t launch_block_first(const double *t, const double *dt, int64_t n, Blo
 cudaError_t launch_block_correct_dev(const JStore &js, const BlockStep &b, int64_t n_max, const double *a1,
                                      const double *j1, double eta, double dt_max, cudaStream_t s) {
     if (n_max <= 0) return cudaSuccess;
-    block_correct_dev_kernel<<<grid_for_warps(n_max), kWarpCta, 0, s>>>(js, b, a1, j1, eta, dt_max);
+    // (most blocks hold a small part of the particles: the grid is capped, and strides)
+    const unsigned g = std::min(grid_for_warps(kLanesPerParticle * n_max), kCorrectMaxCtas);
+    block_correct_dev_kernel<<<g, kWarpCta, 0, s>>>(js, b, a1, j1, eta, dt_max);
     return cudaGetLastError();
 }
 
