@@ -260,7 +260,7 @@ Grouping grouping(const sp2_ctx *c, int kind, int64_t n_i, int64_t n_j) {
 
 // Dynamic shared memory of a pass launch (defined below).
 size_t pass_smem_bytes(int kind, int order, int mixed, int tile, int rb, int threads, int ipt, int fused,
-                       int fused_stages);
+                       int fused_stages, int pair_pad);
 
 // Default launch shape: the one with the smallest estimated time among the CTA
 // forms below (mixed: within the lanes, tile and groups of grouping()).  The
@@ -314,7 +314,8 @@ sp2_launch heuristic(const sp2_ctx *c, int kind, int order, int mixed, int64_t n
                 const int warps = ipt == 1 ? R.warps[0] : fused ? 8 : order == 4 && !nn ? 12 : R.warps[1];
                 for (int tile = mixed ? g.tile : std::max(64, 8 * jl); tile <= (mixed ? g.tile : 512); tile *= 2) {
                     const int64_t unit = mixed ? g.group : tile;
-                    const size_t smem = pass_smem_bytes(kind, order, mixed, tile, rb, threads, ipt, fused, 2);
+                    const size_t smem = pass_smem_bytes(kind, order, mixed, tile, rb, threads, ipt, fused, 2,
+                                                        ipt == 1 && jl >= kPairPadMinLanes ? kPairPad : 0);
                     const int64_t occ = std::min<int64_t>(std::max(1, warps * 32 / threads),
                                                           static_cast<int64_t>(kSmemPerSm / (smem + 2048)));
                     if (occ < 1) continue;
@@ -372,12 +373,22 @@ struct PassOut {
 // pair records, and for the mixed policies the 8-byte running totals of every
 // (thread, sink, field).
 size_t pass_smem_bytes(int kind, int order, int mixed, int tile, int rb, int threads, int ipt, int fused,
-                       int fused_stages) {
+                       int fused_stages, int pair_pad) {
     const size_t ring = fused ? static_cast<size_t>(fused_stages) * tile * 16 * dscache_words(order)
                               : static_cast<size_t>(kStagesDevice) * tile * rb;
-    const size_t pairs = mixed ? static_cast<size_t>(tile) * rb : 0;  // both mixed policies evaluate source pairs
+    const size_t pairs = mixed ? static_cast<size_t>(tile / 2) * (2 * rb + pair_pad) : 0;  // both mixed policies evaluate source pairs
     const int ns = (kind == K_VJP) ? 7 : (order == 6 ? 10 : (order == 2 ? 4 : 7));
     return ring + pairs + (mixed ? static_cast<size_t>(threads) * ipt * ns * 8 : 0);
+}
+
+// Many lanes that share a sink read padded pair records (kPairPad), where they fit.
+int pair_pad_for(int kind, int order, int mixed, int tile, int rb, int threads, int ipt, int jl, int fused,
+                 int fused_stages) {
+    if (!mixed || ipt != 1 || jl < kPairPadMinLanes) return 0;
+    return pass_smem_bytes(kind, order, mixed, tile, rb, threads, ipt, fused, fused_stages, kPairPad) <=
+                   static_cast<size_t>(kMaxPassSmem)
+               ? kPairPad
+               : 0;
 }
 
 // The shape of a pass: the tuned one for the bucket of its sizes, else the
@@ -439,13 +450,15 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
     // fused: two bulk-copy stages when they fit and a slice spans several
     // tiles, else one (the next tile's copy then starts after this one's
     // prediction)
-    const bool two_fit = pass_smem_bytes(kind, order, mixed, tile, rb, L.threads, L.i_per_thread, 1, 2) <=
+    const bool two_fit = pass_smem_bytes(kind, order, mixed, tile, rb, L.threads, L.i_per_thread, 1, 2, 0) <=
                          static_cast<size_t>(kMaxPassSmem);
     const int fused_stages = (fused && (slice_len <= tile || !two_fit)) ? 1 : kFusedStagesDevice;
     key.fused_stages = fused ? fused_stages : 0;
     key.mw = jl > 32 ? 1 : 0;
+    key.pair_pad = pair_pad_for(kind, order, mixed, tile, rb, L.threads, L.i_per_thread, devn ? 32 : jl, fused,
+                                fused_stages);
     const size_t smem_total = pass_smem_bytes(kind, order, mixed, tile, rb, L.threads, L.i_per_thread, fused,
-                                              fused_stages);
+                                              fused_stages, key.pair_pad);
     if (smem_total > static_cast<size_t>(kMaxPassSmem))
         return fail(c, SP2_ERR_UNSUPPORTED, "launch shape needs %zu bytes of shared memory (max %d)", smem_total,
                     kMaxPassSmem);
@@ -515,6 +528,7 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
     p.acc = o.acc; p.jerk = o.jerk; p.snap = o.snap; p.pot = o.pot; p.nn_id = o.nn_id; p.nn_r2 = o.nn_r2;
     p.xbar = o.xbar; p.vbar = o.vbar; p.mbar = o.mbar; p.accumulate = o.accumulate;
     p.sink_rec = o.sink_rec;
+    p.pair_pad = key.pair_pad;
     if (nb) {
         p.nb_h2 = o.nb_h2;
         p.nb_count = o.nb_count;
@@ -1360,6 +1374,7 @@ static sp2_status block_run_impl(sp2_ctx *c, double t_end, double eta, double et
     while (L.split_j > 1 && static_cast<double>(n) * fields * 8.0 * L.split_j > 256.0 * (1 << 20)) L.split_j /= 2;
     {
         KernelKey key{K_FORCE, order, mixed, 0, 1, 0, 0, 1};
+        key.pair_pad = mixed ? kPairPad : 0;
         int per_sm = 0;
         SP2_CK(c, force_kernel_occupancy(key, L.threads, L.j_tile, &per_sm));
         if (per_sm <= 0) return fail(c, SP2_ERR_UNSUPPORTED, "block-step pass does not fit on an SM");
@@ -1549,11 +1564,13 @@ sp2_status sp2_autotune(sp2_ctx *c, int64_t n_i, sp2_launch *best) {
         KernelKey key{K_FORCE, order, mixed, nn, L.i_per_thread, fused};
         key.mw = L.j_lanes > 32 ? 1 : 0;
         // a fused pass that cannot hold two bulk-copy stages runs with one
-        if (fused && pass_smem_bytes(K_FORCE, order, mixed, L.j_tile, c->rb, L.threads, L.i_per_thread, 1, 2) >
+        if (fused && pass_smem_bytes(K_FORCE, order, mixed, L.j_tile, c->rb, L.threads, L.i_per_thread, 1, 2, 0) >
                          static_cast<size_t>(kMaxPassSmem))
             key.fused_stages = 1;
+        key.pair_pad = pair_pad_for(K_FORCE, order, mixed, L.j_tile, c->rb, L.threads, L.i_per_thread, L.j_lanes,
+                                    fused, key.fused_stages ? key.fused_stages : 2);
         if (pass_smem_bytes(K_FORCE, order, mixed, L.j_tile, c->rb, L.threads, L.i_per_thread, fused,
-                            key.fused_stages ? key.fused_stages : 2) > static_cast<size_t>(kMaxPassSmem) ||
+                            key.fused_stages ? key.fused_stages : 2, key.pair_pad) > static_cast<size_t>(kMaxPassSmem) ||
             force_kernel_occupancy(key, L.threads, L.j_tile, &occ) != cudaSuccess) {
             cudaGetLastError();
             return 0;

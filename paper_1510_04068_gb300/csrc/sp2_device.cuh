@@ -1403,7 +1403,7 @@ __device__ __forceinline__ typename P::Rec filler_rec() {
 // record whole; positions past cnt become filler records.
 template <class P>
 __device__ __forceinline__ void predict_staged_tile(const ForceParams &p, const float4 *raw, int cnt,
-                                                    unsigned char *q, int jl) {
+                                                    unsigned char *q, int jl, int prb) {
     constexpr int RW = P::kRawWords;
     constexpr int W = P::RB / 16;
     const int npair = p.tile >> 1;
@@ -1423,7 +1423,7 @@ __device__ __forceinline__ void predict_staged_tile(const ForceParams &p, const 
         P::predict_raw2(wa, wb, p.t_hi, p.t_lo, ra, rb);
         if (a >= cnt) ra = filler_rec<P>();
         if (b >= cnt) rb = filler_rec<P>();
-        unsigned char *d = q + static_cast<size_t>(pr) * P::PRB;
+        unsigned char *d = q + static_cast<size_t>(pr) * prb;
 #pragma unroll
         for (int w = 0; w < W; ++w) P::store_pair_word(ra.w[w], rb.w[w], w, d);
     }
@@ -1432,28 +1432,28 @@ __device__ __forceinline__ void predict_staged_tile(const ForceParams &p, const 
 // Re-lay a staged tile of natural records as pair records: lane lj's sources
 // m = 2k and 2k+1 (tile positions lj + jl*m) form pair k*jl + lj.
 template <class P>
-__device__ __forceinline__ void pair_tile(const unsigned char *st, unsigned char *q, int tile, int jl) {
+__device__ __forceinline__ void pair_tile(const unsigned char *st, unsigned char *q, int tile, int jl, int prb) {
     constexpr int W = P::RB / 16;
     const int items = (tile >> 1) * W;
     for (int i = threadIdx.x; i < items; i += blockDim.x) {
         const int pr = i / W, w = i - pr * W;
         const int k = pr / jl, lj = pr - k * jl;
         const int a = lj + 2 * k * jl;
-        P::pack_word(st + a * P::RB, st + (a + jl) * P::RB, w, q + pr * P::PRB);
+        P::pack_word(st + a * P::RB, st + (a + jl) * P::RB, w, q + pr * prb);
     }
 }
 
 template <class P, int IPT, bool SELF>
-__device__ __forceinline__ void tile_loop(const unsigned char *st, int tb, int per, int jl, int lj,
+__device__ __forceinline__ void tile_loop(const unsigned char *st, int tb, int per, int jl, int lj, int prb,
                                           const typename P::Sink *sk, typename P::Acc *ac,
                                           typename P::real eps2) {
     const unsigned char *base = st + lj * P::RB;
     const int step = jl * P::RB;
     if constexpr (is_paired<P>::value) {
-        // st holds pair records: lane lj's k-th pair (its sources 2k and 2k+1)
-        // sits at pair index k * jl + lj.
-        const unsigned char *pbase = st + lj * P::PRB;
-        const int pstep = jl * P::PRB;
+        // st holds pair records (prb bytes apart): lane lj's k-th pair (its
+        // sources 2k and 2k+1) sits at pair index k * jl + lj.
+        const unsigned char *pbase = st + lj * prb;
+        const int pstep = jl * prb;
         for (int q0 = 0; q0 < per; q0 += P::kChunk) {
             const int jb = tb + q0 * jl + lj;
             const unsigned char *pq = pbase + (q0 >> 1) * pstep;
@@ -1737,8 +1737,11 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
     // fused: one stage when a slice fits one tile, else two
     const int nstage = FUSED ? p.fused_stages : kStages;
     const size_t ring_stride = static_cast<size_t>(p.tile) * (FUSED ? kRaw * 16 : P::RB);
-    unsigned char *pbuf = smem + nstage * ring_stride;  // pair records (kPair)
-    double *tot = reinterpret_cast<double *>(pbuf + (kPair ? static_cast<size_t>(p.tile) * P::RB : 0)) + tid;
+    // pair records (kPair), prb bytes each: padded only in the kernels with one
+    // sink per thread, where many lanes may share a sink (kPairPad)
+    unsigned char *pbuf = smem + nstage * ring_stride;
+    const int prb = 2 * P::RB + (kPair && IPT == 1 ? p.pair_pad : 0);
+    double *tot = reinterpret_cast<double *>(pbuf + (kPair ? static_cast<size_t>(p.tile >> 1) * prb : 0)) + tid;
 
     // fused prediction: one completion barrier per ring stage; bit s of
     // `phase` is the parity of stage s's next completion
@@ -1879,7 +1882,7 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
                 }
                 phase ^= 1u << stage;
                 const int cnt = (tb + p.tile < j1) ? p.tile : static_cast<int>(j1 - tb);
-                predict_staged_tile<P>(p, reinterpret_cast<const float4 *>(smem + stage * ring_stride), cnt, pbuf, jl);
+                predict_staged_tile<P>(p, reinterpret_cast<const float4 *>(smem + stage * ring_stride), cnt, pbuf, jl, prb);
                 if constexpr (P::kCanFuse) {
                     if (t == 0 && !p.sink_rec) {
 #pragma unroll
@@ -1901,7 +1904,7 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
                 st = smem + (t % kStages) * ring_stride;
                 if constexpr (kPair) {
                     // every thread has left the previous tile's pair records (barrier above)
-                    pair_tile<P>(st, pbuf, p.tile, jl);
+                    pair_tile<P>(st, pbuf, p.tile, jl, prb);
                     __syncthreads();
                     st = pbuf;
                 }
@@ -1914,9 +1917,9 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
             // holds) skips the tile and leaves the issue slots to the others
             if (warp_busy) {
                 // the group's part: c0 .. c0 + per * jl, whose (pair) records start c0 records in
-                const unsigned char *sg = st + static_cast<size_t>(c0) * P::RB;
-                if (__any_sync(kFull, mine)) tile_loop<P, IPT, true>(sg, tb + c0, per, jl, lj, sk, ac, eps2);
-                else tile_loop<P, IPT, false>(sg, tb + c0, per, jl, lj, sk, ac, eps2);
+                const unsigned char *sg = st + static_cast<size_t>(c0 >> 1) * prb;
+                if (__any_sync(kFull, mine)) tile_loop<P, IPT, true>(sg, tb + c0, per, jl, lj, prb, sk, ac, eps2);
+                else tile_loop<P, IPT, false>(sg, tb + c0, per, jl, lj, prb, sk, ac, eps2);
             }
             since_flush += per;
             if (since_flush >= P::kFlush || (p.group_tiles > 0 && (t + 1) % p.group_tiles == 0)) {
@@ -2281,9 +2284,9 @@ __global__ void __launch_bounds__(kMaxThreads) batched_kernel(const BatchParams 
 // policies) and, for the mixed policies, the totals of every (thread, sink,
 // field).  The launch and occupancy helpers take the tile, not bytes.
 template <class P, int IPT, bool FUSED>
-inline size_t pass_smem(size_t tile, int threads, int fused_stages = kFusedStages) {
+inline size_t pass_smem(size_t tile, int threads, int fused_stages, int pair_pad) {
     const size_t ring = FUSED ? fused_stages * tile * raw_words<P>::value * 16 : kStages * tile * P::RB;
-    const size_t pair_bytes = is_paired<P>::value ? tile * P::RB : 0;
+    const size_t pair_bytes = is_paired<P>::value ? tile / 2 * (2 * P::RB + pair_pad) : 0;
     return ring + pair_bytes + (P::kSmemTotals ? static_cast<size_t>(threads) * IPT * P::NS * sizeof(double) : 0);
 }
 
@@ -2292,7 +2295,7 @@ constexpr int kMaxDynSmem = kMaxPassSmem;
 template <class P, int IPT, bool FUSED, int DEVN = 0>
 inline cudaError_t launch_pass(const ForceParams &p, int grid, int threads, size_t tile, cudaStream_t s) {
     static bool attr_set = false;
-    const size_t smem = pass_smem<P, IPT, FUSED>(tile, threads, p.fused_stages);
+    const size_t smem = pass_smem<P, IPT, FUSED>(tile, threads, p.fused_stages, p.pair_pad);
     if (smem > static_cast<size_t>(kMaxDynSmem)) return cudaErrorInvalidConfiguration;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(pass_kernel<P, IPT, FUSED, DEVN>,
@@ -2305,8 +2308,9 @@ inline cudaError_t launch_pass(const ForceParams &p, int grid, int threads, size
 }
 
 template <class P, int IPT, bool FUSED, int DEVN = 0>
-inline cudaError_t occupancy_pass(int threads, size_t tile, int *blocks, int fused_stages = 0) {
-    const size_t smem = pass_smem<P, IPT, FUSED>(tile, threads, fused_stages > 0 ? fused_stages : kFusedStages);
+inline cudaError_t occupancy_pass(int threads, size_t tile, int *blocks, const KernelKey &key) {
+    const size_t smem = pass_smem<P, IPT, FUSED>(tile, threads, key.fused_stages > 0 ? key.fused_stages : kFusedStages,
+                                                 key.pair_pad);
     if (smem > static_cast<size_t>(kMaxDynSmem)) {
         *blocks = 0;
         return cudaSuccess;
@@ -2330,71 +2334,71 @@ struct takes_device_count<MixedPairForce<6, false>> { static constexpr bool valu
 template <>
 struct takes_device_count<Fp64Force<6, false>> { static constexpr bool value = true; };
 
+template <class P, int IPT, bool FUSED, int DEVN = 0>
+inline cudaError_t run_or_query(bool occ, const KernelKey &key, const ForceParams *p, int grid, int threads, size_t tile,
+                                cudaStream_t s, int *blocks) {
+    return occ ? occupancy_pass<P, IPT, FUSED, DEVN>(threads, tile, blocks, key)
+               : launch_pass<P, IPT, FUSED, DEVN>(*p, grid, threads, tile, s);
+}
+
 template <class P, bool FUSED>
-inline cudaError_t dispatch_ipt_f(bool occ, int ipt, const ForceParams *p, int grid, int threads, size_t tile,
-                                  cudaStream_t s, int *blocks, int fstages = 0, int mw = 0) {
-    if (mw) {  // several warps per sink: one sink per thread, paired force policies
+inline cudaError_t dispatch_ipt_f(bool occ, const KernelKey &key, const ForceParams *p, int grid, int threads,
+                                  size_t tile, cudaStream_t s, int *blocks) {
+    if (key.mw) {  // several warps per sink: one sink per thread, paired force policies
         if constexpr (shares_sinks<P>::value) {
-            if (ipt != 1) return cudaErrorInvalidValue;
-            return occ ? occupancy_pass<P, 1, FUSED, 2>(threads, tile, blocks, fstages)
-                       : launch_pass<P, 1, FUSED, 2>(*p, grid, threads, tile, s);
+            if (key.ipt != 1) return cudaErrorInvalidValue;
+            return run_or_query<P, 1, FUSED, 2>(occ, key, p, grid, threads, tile, s, blocks);
         } else {
             return cudaErrorInvalidValue;
         }
     }
-    switch (ipt) {
-        case 1: return occ ? occupancy_pass<P, 1, FUSED>(threads, tile, blocks, fstages) : launch_pass<P, 1, FUSED>(*p, grid, threads, tile, s);
-        case 2: return occ ? occupancy_pass<P, 2, FUSED>(threads, tile, blocks, fstages) : launch_pass<P, 2, FUSED>(*p, grid, threads, tile, s);
-        case 4: return occ ? occupancy_pass<P, 4, FUSED>(threads, tile, blocks, fstages) : launch_pass<P, 4, FUSED>(*p, grid, threads, tile, s);
+    switch (key.ipt) {
+        case 1: return run_or_query<P, 1, FUSED>(occ, key, p, grid, threads, tile, s, blocks);
+        case 2: return run_or_query<P, 2, FUSED>(occ, key, p, grid, threads, tile, s, blocks);
+        case 4: return run_or_query<P, 4, FUSED>(occ, key, p, grid, threads, tile, s, blocks);
         default: return cudaErrorInvalidValue;
     }
 }
 
 // fused = 1 is available for the mixed force policies only
 template <class P>
-inline cudaError_t dispatch_ipt(bool occ, int ipt, const ForceParams *p, int grid, int threads, size_t tile,
-                                cudaStream_t s, int *blocks, int fused = 0, int devn = 0, int fstages = 0,
-                                int mw = 0) {
+inline cudaError_t dispatch_ipt(bool occ, const KernelKey &key, const ForceParams *p, int grid, int threads,
+                                size_t tile, cudaStream_t s, int *blocks) {
     if constexpr (takes_device_count<P>::value) {
-        if (devn) {
-            if (ipt != 1 || fused || mw) return cudaErrorInvalidValue;
-            return occ ? occupancy_pass<P, 1, false, 1>(threads, tile, blocks)
-                       : launch_pass<P, 1, false, 1>(*p, grid, threads, tile, s);
+        if (key.devn) {
+            if (key.ipt != 1 || key.fused || key.mw) return cudaErrorInvalidValue;
+            return run_or_query<P, 1, false, 1>(occ, key, p, grid, threads, tile, s, blocks);
         }
     } else {
-        if (devn) return cudaErrorInvalidValue;
+        if (key.devn) return cudaErrorInvalidValue;
     }
     if constexpr (P::kCanFuse && is_paired<P>::value) {
-        if (fused) return dispatch_ipt_f<P, true>(occ, ipt, p, grid, threads, tile, s, blocks, fstages, mw);
+        if (key.fused) return dispatch_ipt_f<P, true>(occ, key, p, grid, threads, tile, s, blocks);
     } else {
-        if (fused) return cudaErrorInvalidValue;
+        if (key.fused) return cudaErrorInvalidValue;
     }
-    return dispatch_ipt_f<P, false>(occ, ipt, p, grid, threads, tile, s, blocks, 0, mw);
+    return dispatch_ipt_f<P, false>(occ, key, p, grid, threads, tile, s, blocks);
 }
 
 // Neighbour-list kernels exist for one sink per thread only.
 template <class P>
-inline cudaError_t dispatch_nb(bool occ, int ipt, const ForceParams *p, int grid, int threads, size_t tile,
-                               cudaStream_t s, int *blocks, int fused, int fstages = 0, int mw = 0) {
-    if (ipt != 1) return cudaErrorInvalidValue;
+inline cudaError_t dispatch_nb(bool occ, const KernelKey &key, const ForceParams *p, int grid, int threads, size_t tile,
+                               cudaStream_t s, int *blocks) {
+    if (key.ipt != 1) return cudaErrorInvalidValue;
     if constexpr (P::kCanFuse && is_paired<P>::value) {
-        if (fused && mw)
-            return occ ? occupancy_pass<P, 1, true, 2>(threads, tile, blocks, fstages)
-                       : launch_pass<P, 1, true, 2>(*p, grid, threads, tile, s);
-        if (fused)
-            return occ ? occupancy_pass<P, 1, true>(threads, tile, blocks, fstages)
-                       : launch_pass<P, 1, true>(*p, grid, threads, tile, s);
+        if (key.fused)
+            return key.mw ? run_or_query<P, 1, true, 2>(occ, key, p, grid, threads, tile, s, blocks)
+                          : run_or_query<P, 1, true>(occ, key, p, grid, threads, tile, s, blocks);
     } else {
-        if (fused) return cudaErrorInvalidValue;
+        if (key.fused) return cudaErrorInvalidValue;
     }
-    if (mw) {
+    if (key.mw) {
         if constexpr (shares_sinks<P>::value)
-            return occ ? occupancy_pass<P, 1, false, 2>(threads, tile, blocks)
-                       : launch_pass<P, 1, false, 2>(*p, grid, threads, tile, s);
+            return run_or_query<P, 1, false, 2>(occ, key, p, grid, threads, tile, s, blocks);
         else
             return cudaErrorInvalidValue;
     }
-    return occ ? occupancy_pass<P, 1, false>(threads, tile, blocks) : launch_pass<P, 1, false>(*p, grid, threads, tile, s);
+    return run_or_query<P, 1, false>(occ, key, p, grid, threads, tile, s, blocks);
 }
 
 template <class P>
@@ -2432,25 +2436,19 @@ inline cudaError_t occupancy_batched(int threads, int *blocks) {
     cudaError_t launch_force_##SUFFIX(const KernelKey &k, const ForceParams &p, int grid, int threads,     \
                                       size_t tile, cudaStream_t s) {                                       \
         if (k.nb)                                                                                          \
-            return k.nn ? dispatch_nb<WithNeighbours<POLICY<ORDER, true>>>(false, k.ipt, &p, grid, threads,  \
-                                                                           tile, s, nullptr, k.fused, 0,   \
-                                                                           k.mw)                           \
+            return k.nn ? dispatch_nb<WithNeighbours<POLICY<ORDER, true>>>(false, k, &p, grid, threads, tile,\
+                                                                           s, nullptr)                     \
                         : cudaErrorInvalidValue;                                                           \
-        return k.nn ? dispatch_ipt<POLICY<ORDER, true>>(false, k.ipt, &p, grid, threads, tile, s, nullptr,  \
-                                                        k.fused, k.devn, 0, k.mw)                          \
-                    : dispatch_ipt<POLICY<ORDER, false>>(false, k.ipt, &p, grid, threads, tile, s, nullptr, \
-                                                         k.fused, k.devn, 0, k.mw);                        \
+        return k.nn ? dispatch_ipt<POLICY<ORDER, true>>(false, k, &p, grid, threads, tile, s, nullptr)     \
+                    : dispatch_ipt<POLICY<ORDER, false>>(false, k, &p, grid, threads, tile, s, nullptr);   \
     }                                                                                                      \
-    cudaError_t occupancy_force_##SUFFIX(const KernelKey &k, int threads, size_t tile, int *blocks) {       \
+    cudaError_t occupancy_force_##SUFFIX(const KernelKey &k, int threads, size_t tile, int *blocks) {      \
         if (k.nb)                                                                                          \
-            return k.nn ? dispatch_nb<WithNeighbours<POLICY<ORDER, true>>>(true, k.ipt, nullptr, 0, threads, \
-                                                                           tile, 0, blocks, k.fused,        \
-                                                                           k.fused_stages, k.mw)            \
+            return k.nn ? dispatch_nb<WithNeighbours<POLICY<ORDER, true>>>(true, k, nullptr, 0, threads, tile,\
+                                                                           0, blocks)                      \
                         : cudaErrorInvalidValue;                                                           \
-        return k.nn ? dispatch_ipt<POLICY<ORDER, true>>(true, k.ipt, nullptr, 0, threads, tile, 0, blocks,  \
-                                                        k.fused, k.devn, k.fused_stages, k.mw)             \
-                    : dispatch_ipt<POLICY<ORDER, false>>(true, k.ipt, nullptr, 0, threads, tile, 0, blocks, \
-                                                         k.fused, k.devn, k.fused_stages, k.mw);           \
+        return k.nn ? dispatch_ipt<POLICY<ORDER, true>>(true, k, nullptr, 0, threads, tile, 0, blocks)     \
+                    : dispatch_ipt<POLICY<ORDER, false>>(true, k, nullptr, 0, threads, tile, 0, blocks);   \
     }                                                                                                      \
     cudaError_t launch_reduce_##SUFFIX(const KernelKey &k, const ForceParams &r, cudaStream_t s) {         \
         return k.nn ? launch_reduce<POLICY<ORDER, true>>(r, s) : launch_reduce<POLICY<ORDER, false>>(r, s); \

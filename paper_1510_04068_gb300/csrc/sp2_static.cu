@@ -147,6 +147,7 @@ extern "C" sp2_status sp2_step_static(int64_t n_j, const int32_t *id, const doub
     if (launch_predict(4, 1, js, n_j, t, rec, s) != cudaSuccess) return SP2_ERR_CUDA;
 
     KernelKey key{K_FORCE, 4, 1, nn, L.i_per_thread};
+    key.pair_pad = L.i_per_thread == 1 && L.j_lanes >= kPairPadMinLanes ? kPairPad : 0;
     int per_sm = 0;
     if (force_kernel_occupancy(key, L.threads, L.j_tile, &per_sm) != cudaSuccess || per_sm <= 0) return SP2_ERR_CUDA;
     ForceParams fp{};
@@ -159,6 +160,7 @@ extern "C" sp2_status sp2_step_static(int64_t n_j, const int32_t *id, const doub
     fp.split = static_cast<int>(split);
     fp.jl = L.j_lanes;
     fp.tile = L.j_tile;
+    fp.pair_pad = key.pair_pad;
     fp.sinks_per_cta = static_cast<int>(sinks_per_cta);
     fp.n_iblk = n_iblk;
     fp.n_items = n_iblk * split;
