@@ -881,7 +881,7 @@ sp2_status sp2_set_j(sp2_ctx *c, int64_t first, int64_t n, const int32_t *slots,
             SP2_CK(c, cudaStreamSynchronize(c->stream));
         } else {
             Staging s{c};
-            s.plan(n * sizeof(int32_t)); s.plan(n * sizeof(int32_t)); s.plan(2 * n * sizeof(double));
+            s.plan(n * sizeof(int32_t)); s.plan(n * sizeof(int32_t)); s.plan(n * sizeof(double)); s.plan(n * sizeof(double));
             s.plan(n3); s.plan(n3); s.plan(n3); s.plan(n3); if (snap) s.plan(n3);
             SP2_CKS(ensure(c, reinterpret_cast<void **>(&c->stage), &c->stage_cap, s.total, "staging"));
             const int32_t *dsl = stage_in(s, slots, n);
