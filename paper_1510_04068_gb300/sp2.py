@@ -10,6 +10,7 @@ in libsapporo_gb.so; if the library cannot be loaded, every call raises.
 from __future__ import annotations
 
 import ctypes
+import sys
 from ctypes import POINTER, Structure, byref, c_char_p, c_double, c_int, c_int32, c_int64, c_size_t, c_void_p
 from pathlib import Path
 
@@ -121,21 +122,23 @@ def _check(status: int, ctx=None):
         raise SP2Error(status, msg or (_lib.sp2_strerror(status) or b"").decode())
 
 
-def _is_torch(a):
-    return type(a).__module__.startswith("torch")
+F8, I4, I8 = np.float64, np.int32, np.int64
+_TORCH_DTYPES = {}  # numpy dtype class -> torch dtype, filled once torch is there
 
 
 def _marshal(arrays, dtypes):
     """Pointers and ptr_kind for a call; all non-None arrays must live together."""
     kinds, ptrs, keep = set(), [], []
+    torch = sys.modules.get("torch")  # no tensor can exist before torch is imported
+    if torch is not None and not _TORCH_DTYPES:
+        _TORCH_DTYPES.update({F8: torch.float64, I4: torch.int32, I8: torch.int64})
     for a, dt in zip(arrays, dtypes):
         if a is None:
             ptrs.append(None)
             continue
-        if _is_torch(a):
-            import torch
-            want = {np.float64: torch.float64, np.int32: torch.int32, np.int64: torch.int64}[dt]
-            if a.dtype != want or not a.is_contiguous():
+        if torch is not None and isinstance(a, torch.Tensor):
+            want = _TORCH_DTYPES[dt]
+            if a.dtype is not want or not a.is_contiguous():
                 raise TypeError(f"tensor must be contiguous {want}, got {a.dtype}")
             kinds.add(SP2_DEVICE if a.is_cuda else SP2_HOST)
             ptrs.append(a.data_ptr())
@@ -148,9 +151,6 @@ def _marshal(arrays, dtypes):
     if len(kinds) > 1:
         raise TypeError("mixing host and device arrays in one call")
     return ptrs, (kinds.pop() if kinds else SP2_HOST), keep
-
-
-F8, I4, I8 = np.float64, np.int32, np.int64
 
 
 def sp2_open(order=4, precision=SP2_MIXED, n_max=1, eps2=0.0, with_nn=1, cuda_stream=None,
