@@ -18,6 +18,7 @@
 
 #include "sp2_ds.cuh"
 #include "sp2_internal.h"
+#include "sp2_launch.cuh"
 
 namespace sp2 {
 
@@ -314,7 +315,7 @@ struct MixedForce {
     __device__ static __forceinline__ Rec ld_global(const unsigned char *p) {
         Rec r;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) r.w[w] = __ldg(reinterpret_cast<const float4 *>(p) + w);
+        for (int w = 0; w < NW; ++w) r.w[w] = ld_plain(reinterpret_cast<const float4 *>(p) + w);
         return r;
     }
     // Far-away, massless filler for the ragged end of a tile: its terms are
@@ -825,7 +826,7 @@ struct Fp64Force {
     __device__ static __forceinline__ Rec ld_global(const unsigned char *p) {
         Rec r;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) r.w[w] = __ldg(reinterpret_cast<const double2 *>(p) + w);
+        for (int w = 0; w < NW; ++w) r.w[w] = ld_plain(reinterpret_cast<const double2 *>(p) + w);
         return r;
     }
     __device__ static __forceinline__ uint4 sentinel(int w) {
@@ -1037,7 +1038,7 @@ struct MixedVjp {
     __device__ static __forceinline__ Rec ld_global(const unsigned char *p) {
         Rec r;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) r.w[w] = __ldg(reinterpret_cast<const float4 *>(p) + w);
+        for (int w = 0; w < NW; ++w) r.w[w] = ld_plain(reinterpret_cast<const float4 *>(p) + w);
         return r;
     }
     __device__ static __forceinline__ uint4 sentinel(int w) {
@@ -1295,7 +1296,7 @@ struct Fp64Vjp {
     __device__ static __forceinline__ Rec ld_global(const unsigned char *p) {
         Rec r;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) r.w[w] = __ldg(reinterpret_cast<const double2 *>(p) + w);
+        for (int w = 0; w < NW; ++w) r.w[w] = ld_plain(reinterpret_cast<const double2 *>(p) + w);
         return r;
     }
     __device__ static __forceinline__ uint4 sentinel(int w) {
@@ -1832,7 +1833,7 @@ __device__ __forceinline__ void pass_body(const ForceParams &p) {
         for (int k = 0; k < IPT; ++k) {
             ii[k] = iblk * p.sinks_per_cta + static_cast<int64_t>(k) * slots + islot;
             val[k] = ii[k] < p.n_i;
-            const int raw = val[k] ? __ldg(p.i_idx + ii[k]) : 0;
+            const int raw = val[k] ? ld_plain(p.i_idx + ii[k]) : 0;
             if (p.sink_rec) {
                 // explicit sink: its own record; raw names its slot for the self pair (< 0: none)
                 if (val[k] && raw >= p.n_loaded) {
@@ -2116,6 +2117,7 @@ struct pass_min_blocks<MixedPairForce<4, true>, 2, false> { static constexpr int
 template <class P, int IPT, bool FUSED, int MODE = 0>
 __global__ void __launch_bounds__(kMaxThreads, (pass_min_blocks<P, IPT, FUSED>::value)) pass_kernel(const ForceParams p) {
     constexpr bool DEVN = MODE == 1;
+    grid_wait();
     if constexpr (MODE == 2) {
         pass_body<P, IPT, FUSED, true>(p);
     } else if constexpr (DEVN) {
@@ -2144,6 +2146,7 @@ template <class P>
 __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const ForceParams p, int groups) {
     __shared__ double s_v[kReduceThreads];
     __shared__ int32_t s_id[kReduceThreads];
+    grid_wait();
     reduce_columns<P>(p, p.tail_sink0, p.n_i - p.tail_sink0,
                       static_cast<int64_t>(blockIdx.x) * (kReduceThreads / groups), groups, s_v, s_id);
 }
@@ -2195,6 +2198,7 @@ __device__ __forceinline__ void batch_tile_loop(const unsigned char *st, int tb,
 template <class P>
 __global__ void __launch_bounds__(kMaxThreads) batched_kernel(const BatchParams b) {
     extern __shared__ __align__(16) unsigned char smem[];
+    grid_wait();
     const int lane = threadIdx.x & 31;
     unsigned char *wbuf = smem + static_cast<size_t>(threadIdx.x >> 5) * kBatchTile * P::RB;
     const typename P::real eps2 = static_cast<typename P::real>(b.eps2);
@@ -2209,7 +2213,7 @@ __global__ void __launch_bounds__(kMaxThreads) batched_kernel(const BatchParams 
     while (item < b.n_items) {
         unsigned next = 0;
         if (lane == 0) next = n_warps + atomicAdd(b.queue, 1u);
-        const int4 it = __ldg(b.items + item);  // {system first slot, size, chunk first slot, chunk size}
+        const int4 it = ld_plain(b.items + item);  // {system first slot, size, chunk first slot, chunk size}
         const bool val = lane < it.w;
         const int slot = it.z + (val ? lane : 0);
         typename P::Sink sk;
@@ -2230,15 +2234,15 @@ __global__ void __launch_bounds__(kMaxThreads) batched_kernel(const BatchParams 
             if constexpr (is_paired<P>::value) {
                 for (int c = lane; c < (padded >> 1) * W; c += 32) {
                     const int pr = c / W, w = c - pr * W;
-                    const uint4 x = (2 * pr < cnt) ? __ldg(tsrc + 2 * pr * W + w) : P::sentinel(w);
-                    const uint4 y = (2 * pr + 1 < cnt) ? __ldg(tsrc + (2 * pr + 1) * W + w) : P::sentinel(w);
+                    const uint4 x = (2 * pr < cnt) ? ld_plain(tsrc + 2 * pr * W + w) : P::sentinel(w);
+                    const uint4 y = (2 * pr + 1 < cnt) ? ld_plain(tsrc + (2 * pr + 1) * W + w) : P::sentinel(w);
                     P::store_pair_word(*reinterpret_cast<const float4 *>(&x), *reinterpret_cast<const float4 *>(&y), w,
                                        wbuf + pr * P::PRB);
                 }
             } else {
                 for (int c = lane; c < padded * W; c += 32) {
                     uint4 w4;
-                    if (c < cnt * W) w4 = __ldg(tsrc + c);
+                    if (c < cnt * W) w4 = ld_plain(tsrc + c);
                     else w4 = P::sentinel(c % W);
                     *reinterpret_cast<uint4 *>(wbuf + 16 * c) = w4;
                 }
@@ -2303,8 +2307,8 @@ inline cudaError_t launch_pass(const ForceParams &p, int grid, int threads, size
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    pass_kernel<P, IPT, FUSED, DEVN><<<grid, threads, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_overlapped(pass_kernel<P, IPT, FUSED, DEVN>, static_cast<unsigned>(grid),
+                             static_cast<unsigned>(threads), smem, s, p);
 }
 
 template <class P, int IPT, bool FUSED, int DEVN = 0>
@@ -2407,8 +2411,8 @@ inline cudaError_t launch_reduce(const ForceParams &p, cudaStream_t s) {
     const int64_t n = NF * (p.n_i - p.tail_sink0);
     const int groups = p.split < kGroupReduceMinSplit ? 1 : n <= kReduceFewColumns ? kReduceGroupsFew : kReduceGroups;
     const int64_t cols = kReduceThreads / groups;
-    reduce_kernel<P><<<static_cast<unsigned>((n + cols - 1) / cols), kReduceThreads, 0, s>>>(p, groups);
-    return cudaGetLastError();
+    return launch_overlapped(reduce_kernel<P>, static_cast<unsigned>((n + cols - 1) / cols), kReduceThreads, 0, s, p,
+                             groups);
 }
 
 template <class P>
@@ -2418,8 +2422,8 @@ inline size_t batched_smem(int threads) {
 
 template <class P>
 inline cudaError_t launch_batched(const BatchParams &b, int grid, int threads, cudaStream_t s) {
-    batched_kernel<P><<<grid, threads, batched_smem<P>(threads), s>>>(b);
-    return cudaGetLastError();
+    return launch_overlapped(batched_kernel<P>, static_cast<unsigned>(grid), static_cast<unsigned>(threads),
+                             batched_smem<P>(threads), s, b);
 }
 
 template <class P>

@@ -8,6 +8,15 @@
 
 namespace sp2 {
 
+// Loads of what an earlier kernel of the stream wrote: plain ones, because the
+// read-only path (ld.global.nc) asks that nothing writes the data while the
+// kernel is resident, and kernels here are brought onto the SMs before their
+// predecessor has completed (sp2_launch.cuh).
+template <class T>
+__device__ __forceinline__ T ld_plain(const T *p) {
+    return *p;
+}
+
 // ---- double-single arithmetic (Dekker 1971; Knuth's TwoSum; TwoProd by FMA).
 // Every step is explicitly rounded so no multiply-add is fused behind our back.
 struct ds {
@@ -75,13 +84,13 @@ __device__ __forceinline__ void ds_fetch(const float4 *dsc, int64_t j, float4 *w
     constexpr int W = (ORDER == 6) ? 8 : 7;
     const float4 *q = dsc + j * W;
     if (ORDER == 2) {
-        w[0] = __ldg(q);
-        w[1] = __ldg(q + 1);
-        w[3] = __ldg(q + 3);
+        w[0] = ld_plain(q);
+        w[1] = ld_plain(q + 1);
+        w[3] = ld_plain(q + 3);
         return;
     }
 #pragma unroll
-    for (int k = 0; k < W; ++k) w[k] = __ldg(q + k);
+    for (int k = 0; k < W; ++k) w[k] = ld_plain(q + k);
 }
 
 // Mixed-precision prediction of a particle from the cache words ds_fetch

@@ -15,6 +15,7 @@
 
 #include "sp2_ds.cuh"
 #include "sp2_internal.h"
+#include "sp2_launch.cuh"
 
 namespace sp2 {
 namespace {
@@ -127,6 +128,7 @@ __device__ __forceinline__ void write_dscache_scalars(const JStore &d, int64_t s
 }
 
 __global__ void __launch_bounds__(kSmallThreads) dscache_kernel(JStore d, int64_t first, int64_t n) {
+    grid_wait();
     const int64_t g = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t s = first + g / kLanesPerParticle;
     const int c = static_cast<int>(g % kLanesPerParticle);
@@ -193,6 +195,7 @@ __device__ __forceinline__ bool block_select(const BlockStep &b, int64_t j, int6
 template <int ORDER, bool BLOCK>
 __global__ void predict_ds_kernel(const float4 *dsc, int64_t n, float t_hi, float t_lo, unsigned char *rec,
                                   const BlockStep b) {
+    grid_wait();
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if constexpr (BLOCK) {
         double t;
@@ -214,6 +217,7 @@ __global__ void __launch_bounds__(kSmallThreads)
 scatter_kernel(JStore d, const int32_t *slots, int64_t n, int64_t n_loaded, unsigned int *err, const int32_t *id,
                const double *m, const double *x, const double *v, const double *a, const double *jk, const double *sn,
                const double *t) {
+    grid_wait();
     const int64_t g = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t k = g / kLanesPerParticle;
     const int c = static_cast<int>(g % kLanesPerParticle);
@@ -248,6 +252,7 @@ scatter_kernel(JStore d, const int32_t *slots, int64_t n, int64_t n_loaded, unsi
 
 template <int ORDER, bool MIXED, bool BLOCK>
 __global__ void predict_kernel(JStore js, int64_t n, double t, unsigned char *rec, const BlockStep b) {
+    grid_wait();
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if constexpr (BLOCK) {
         if (!block_select(b, j, n, &t)) return;
@@ -304,6 +309,7 @@ __global__ void predict_kernel(JStore js, int64_t n, double t, unsigned char *re
 
 template <bool MIXED>
 __global__ void pack_state_kernel(int64_t n, const double *m, const double *x, const double *v, unsigned char *rec) {
+    grid_wait();
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const double xp[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
@@ -325,6 +331,7 @@ constexpr int kNbWarps = 4;
 
 __global__ void __launch_bounds__(32 * kNbWarps)
 nb_finish_kernel(const int32_t *ids, int64_t n_i, int nb_max, const int32_t *count, int32_t *list) {
+    grid_wait();
     __shared__ int32_t buf[kNbWarps][kNbShared];
     const int lane = threadIdx.x & 31;
     const int64_t i = static_cast<int64_t>(blockIdx.x) * kNbWarps + (threadIdx.x >> 5);
@@ -517,6 +524,7 @@ __device__ __forceinline__ void count_block(BlockDev *bd, unsigned int n_act, do
 
 __global__ void __launch_bounds__(kWarpCta)
 block_correct_dev_kernel(JStore js, const BlockStep b, const double *a1, const double *j1, double eta, double dt_max) {
+    grid_wait();
     constexpr int kPer = kWarpCta / kLanesPerParticle;  // particles of a CTA (one warp) at a time
     const unsigned int n_act = b.bd->count[b.slot];
     const double t1 = key_time(b.bd->t1bits[b.slot]);
@@ -616,6 +624,7 @@ __global__ void iota_kernel(int32_t *dst, int64_t n) {
 template <bool MIXED>
 __global__ void h4_predict_pack_kernel(int64_t n, double dt, const double *m, const double *x, const double *v,
                                        const double *a, const double *jk, unsigned char *rec) {
+    grid_wait();
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const double h2 = dt * dt * 0.5, h3 = dt * dt * dt * (1.0 / 6.0);
@@ -632,6 +641,7 @@ __global__ void h4_predict_pack_kernel(int64_t n, double dt, const double *m, co
 // Hermite-4 corrector (Makino & Aarseth 1992), in place; a1, j1 at the predicted state.
 __global__ void h4_correct_kernel(int64_t n3, double dt, double *x, double *v, double *a, double *jk,
                                   const double *a1, const double *j1) {
+    grid_wait();
     const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (q >= n3) return;
     const double h = 0.5 * dt, h12 = dt * dt / 12.0;
@@ -672,6 +682,7 @@ __device__ __forceinline__ void store_vjp(bool mixed, unsigned char *rec, int64_
 template <bool MIXED>
 __global__ void pack_vjp_kernel(int64_t n, const double *m, const double *x, const double *v, const double *abar,
                                 const double *jbar, const double *pbar, unsigned char *rec) {
+    grid_wait();
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const double zero[3] = {0.0, 0.0, 0.0};
@@ -688,6 +699,7 @@ template <bool MIXED>
 __global__ void h4_vjp_pre_kernel(int64_t n, double dt, const double *m, const double *x, const double *v,
                                   const double *a, const double *jk, const double *gx, const double *gv,
                                   const double *ga, const double *gj, unsigned char *rec) {
+    grid_wait();
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const double h2 = dt * dt * 0.5, h3 = dt * dt * dt * (1.0 / 6.0), h12 = dt * dt / 12.0;
@@ -707,6 +719,7 @@ __global__ void h4_vjp_pre_kernel(int64_t n, double dt, const double *m, const d
 // force VJP (xpbar, vpbar) at the predicted state.
 __global__ void h4_vjp_post_kernel(int64_t n3, double dt, const double *xpbar, const double *vpbar, double *gx,
                                    double *gv, double *ga, double *gj) {
+    grid_wait();
     const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (q >= n3) return;
     const double h = 0.5 * dt, h2 = dt * dt * 0.5, h3 = dt * dt * dt * (1.0 / 6.0), h12 = dt * dt / 12.0;
@@ -730,14 +743,14 @@ cudaError_t launch_scatter_j(const JStore &dst, const int32_t *slots, int64_t n,
                              const int32_t *id, const double *m, const double *x, const double *v, const double *a,
                              const double *jk, const double *sn, const double *t, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    scatter_kernel<<<grid_for_store(n), kSmallThreads, 0, s>>>(dst, slots, n, n_loaded, err, id, m, x, v, a, jk, sn, t);
+    launch_overlapped(scatter_kernel, grid_for_store(n), kSmallThreads, 0, s, dst, slots, n, n_loaded, err, id, m, x, v, a, jk, sn, t);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dscache(int order, const JStore &js, int64_t first, int64_t n, cudaStream_t s) {
     if (n <= 0 || !js.dsc) return cudaSuccess;
     (void)order;
-    dscache_kernel<<<grid_for_store(n), kSmallThreads, 0, s>>>(js, first, n);
+    launch_overlapped(dscache_kernel, grid_for_store(n), kSmallThreads, 0, s, js, first, n);
     return cudaGetLastError();
 }
 
@@ -749,22 +762,22 @@ cudaError_t launch_predict_form(int order, int mixed, const JStore &js, int64_t 
     if (mixed && js.dsc) {
         const float th = static_cast<float>(t);
         const float tl = static_cast<float>(t - static_cast<double>(th));
-        if (order == 6) predict_ds_kernel<6, BLOCK><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, b);
-        else if (order == 2) predict_ds_kernel<2, BLOCK><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, b);
-        else predict_ds_kernel<4, BLOCK><<<g, kThreads, 0, s>>>(js.dsc, n, th, tl, rec, b);
+        if (order == 6) launch_overlapped(predict_ds_kernel<6, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
+        else if (order == 2) launch_overlapped(predict_ds_kernel<2, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
+        else launch_overlapped(predict_ds_kernel<4, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
         return cudaGetLastError();
     }
     // the FP64 predictor is FP64-bound: 64-thread CTAs spread it over the SMs
     const unsigned g64 = static_cast<unsigned>((n + 63) / 64);
     if (order == 6) {
-        if (mixed) predict_kernel<6, true, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
-        else predict_kernel<6, false, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
+        if (mixed) launch_overlapped(predict_kernel<6, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        else launch_overlapped(predict_kernel<6, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
     } else if (order == 2) {
-        if (mixed) predict_kernel<2, true, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
-        else predict_kernel<2, false, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
+        if (mixed) launch_overlapped(predict_kernel<2, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        else launch_overlapped(predict_kernel<2, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
     } else {
-        if (mixed) predict_kernel<4, true, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
-        else predict_kernel<4, false, BLOCK><<<g64, 64, 0, s>>>(js, n, t, rec, b);
+        if (mixed) launch_overlapped(predict_kernel<4, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        else launch_overlapped(predict_kernel<4, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
     }
     return cudaGetLastError();
 }
@@ -785,8 +798,8 @@ cudaError_t launch_block_predict(int order, int mixed, const JStore &js, int64_t
 cudaError_t launch_pack_state(int mixed, int64_t n, const double *m, const double *x, const double *v,
                               unsigned char *rec, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (mixed) pack_state_kernel<true><<<grid_small(n), kSmallThreads, 0, s>>>(n, m, x, v, rec);
-    else pack_state_kernel<false><<<grid_small(n), kSmallThreads, 0, s>>>(n, m, x, v, rec);
+    if (mixed) launch_overlapped(pack_state_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, rec);
+    else launch_overlapped(pack_state_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, rec);
     return cudaGetLastError();
 }
 
@@ -821,7 +834,7 @@ cudaError_t launch_block_correct_dev(const JStore &js, const BlockStep &b, int64
     if (n_max <= 0) return cudaSuccess;
     // (most blocks hold a small part of the particles: the grid is capped, and strides)
     const unsigned g = std::min(grid_for_warps(kLanesPerParticle * n_max), kCorrectMaxCtas);
-    block_correct_dev_kernel<<<g, kWarpCta, 0, s>>>(js, b, a1, j1, eta, dt_max);
+    launch_overlapped(block_correct_dev_kernel, g, kWarpCta, 0, s, js, b, a1, j1, eta, dt_max);
     return cudaGetLastError();
 }
 
@@ -843,7 +856,7 @@ cudaError_t launch_block_init(const JStore &js, double *dt, int64_t n, double et
 cudaError_t launch_nb_finish(const int32_t *ids, int64_t n_i, int nb_max, const int32_t *count, int32_t *list,
                              cudaStream_t s) {
     if (n_i <= 0) return cudaSuccess;
-    nb_finish_kernel<<<static_cast<unsigned>((n_i + kNbWarps - 1) / kNbWarps), 32 * kNbWarps, 0, s>>>(ids, n_i, nb_max, count, list);
+    launch_overlapped(nb_finish_kernel, static_cast<unsigned>((n_i + kNbWarps - 1) / kNbWarps), 32 * kNbWarps, 0, s, ids, n_i, nb_max, count, list);
     return cudaGetLastError();
 }
 
@@ -851,15 +864,15 @@ cudaError_t launch_h4_predict_pack(int mixed, int64_t n, double dt, const double
                                    const double *v, const double *a, const double *jk, unsigned char *rec,
                                    cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (mixed) h4_predict_pack_kernel<true><<<grid_small(n), kSmallThreads, 0, s>>>(n, dt, m, x, v, a, jk, rec);
-    else h4_predict_pack_kernel<false><<<grid_small(n), kSmallThreads, 0, s>>>(n, dt, m, x, v, a, jk, rec);
+    if (mixed) launch_overlapped(h4_predict_pack_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, rec);
+    else launch_overlapped(h4_predict_pack_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, rec);
     return cudaGetLastError();
 }
 
 cudaError_t launch_h4_correct(int64_t n, double dt, double *x, double *v, double *a, double *jk, const double *a1,
                               const double *j1, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    h4_correct_kernel<<<grid_small(3 * n), kSmallThreads, 0, s>>>(3 * n, dt, x, v, a, jk, a1, j1);
+    launch_overlapped(h4_correct_kernel, grid_small(3 * n), kSmallThreads, 0, s, 3 * n, dt, x, v, a, jk, a1, j1);
     return cudaGetLastError();
 }
 
@@ -867,15 +880,15 @@ cudaError_t launch_h4_vjp_pre(int mixed, int64_t n, double dt, const double *m, 
                               const double *a, const double *jk, const double *gx, const double *gv,
                               const double *ga, const double *gj, unsigned char *vrec, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (mixed) h4_vjp_pre_kernel<true><<<grid_small(n), kSmallThreads, 0, s>>>(n, dt, m, x, v, a, jk, gx, gv, ga, gj, vrec);
-    else h4_vjp_pre_kernel<false><<<grid_small(n), kSmallThreads, 0, s>>>(n, dt, m, x, v, a, jk, gx, gv, ga, gj, vrec);
+    if (mixed) launch_overlapped(h4_vjp_pre_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, gx, gv, ga, gj, vrec);
+    else launch_overlapped(h4_vjp_pre_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, gx, gv, ga, gj, vrec);
     return cudaGetLastError();
 }
 
 cudaError_t launch_h4_vjp_post(int64_t n, double dt, const double *xpbar, const double *vpbar, double *gx,
                                double *gv, double *ga, double *gj, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    h4_vjp_post_kernel<<<grid_small(3 * n), kSmallThreads, 0, s>>>(3 * n, dt, xpbar, vpbar, gx, gv, ga, gj);
+    launch_overlapped(h4_vjp_post_kernel, grid_small(3 * n), kSmallThreads, 0, s, 3 * n, dt, xpbar, vpbar, gx, gv, ga, gj);
     return cudaGetLastError();
 }
 
@@ -883,8 +896,8 @@ cudaError_t launch_pack_vjp(int mixed, int64_t n, const double *m, const double 
                             const double *abar, const double *jbar, const double *pbar, unsigned char *vrec,
                             cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (mixed) pack_vjp_kernel<true><<<grid_small(n), kSmallThreads, 0, s>>>(n, m, x, v, abar, jbar, pbar, vrec);
-    else pack_vjp_kernel<false><<<grid_small(n), kSmallThreads, 0, s>>>(n, m, x, v, abar, jbar, pbar, vrec);
+    if (mixed) launch_overlapped(pack_vjp_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, abar, jbar, pbar, vrec);
+    else launch_overlapped(pack_vjp_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, abar, jbar, pbar, vrec);
     return cudaGetLastError();
 }
 
