@@ -1711,17 +1711,14 @@ sp2_status sp2_autotune(sp2_ctx *c, int64_t n_i, sp2_launch *best) {
                     shapes.push_back({ms, L});
                 }
             }
-    {
-        float ms = 0.f;
-        if (time_shape(h, 1, &ms) == SP2_OK) shapes.push_back({ms, h});
-    }
-    if (shapes.empty()) return fail(c, SP2_ERR_UNSUPPORTED, "no launch shape could run");
     std::sort(shapes.begin(), shapes.end(), [](const std::pair<float, sp2_launch> &x, const std::pair<float, sp2_launch> &y) {
         return x.first < y.first;
     });
-    // stage 2: the best shapes over 1 .. 16 waves, three timed runs each
-    std::vector<sp2_launch> cand;
-    for (size_t r = 0; r < std::min<size_t>(4, shapes.size()); ++r) {
+    // stage 2: the default shape as it is and the best shapes over 1 .. 16 waves,
+    // three timed runs each (the default is not ranked in stage 1: its split is
+    // chosen already, which would put it before forms that gain more from theirs)
+    std::vector<sp2_launch> cand{h};
+    for (size_t r = 0; r < std::min<size_t>(8, shapes.size()); ++r) {
         const sp2_launch base = shapes[r].second;
         const int occ = occupancy(base);
         cand.push_back(base);
@@ -1742,6 +1739,7 @@ sp2_status sp2_autotune(sp2_ctx *c, int64_t n_i, sp2_launch *best) {
         if (st != SP2_OK) return st;
         if (ms < best_ms) { best_ms = ms; best_k = k; }
     }
+    if (best_ms >= 1e30f) return fail(c, SP2_ERR_UNSUPPORTED, "no launch shape could run");
     c->tuned[tune_key(n_i, n_j)] = cand[best_k];
     if (best) *best = cand[best_k];
     return SP2_OK;
