@@ -46,12 +46,11 @@ struct sp2_batch_plan {
     int64_t max_size = 0;
 };
 
-// A pinned buffer of the host-pointer calls; ev: the last copy out of it.
+// The pinned buffer of the host-pointer calls; busy: a copy out of it may be under way.
 struct HostStage {
     unsigned char *buf = nullptr;
     size_t cap = 0;
-    cudaEvent_t ev = nullptr;
-    bool pending = false;
+    bool busy = false;
 };
 
 struct sp2_ctx {
@@ -95,8 +94,7 @@ struct sp2_ctx {
     bool blk_ready = false;                 // sp2_block_init has run since the last set_j
     unsigned char *stage = nullptr;  // staging for host-pointer calls
     size_t stage_cap = 0;
-    HostStage hstage[2];             // its pinned images (host_stage)
-    int hstage_next = 0;
+    HostStage hstage;                // its pinned image (host_stage)
     std::vector<void *> owned;       // everything allocated (for close)
 
     std::map<int64_t, sp2_launch> tuned;  // key: tune_key(n_i, n_j)
@@ -662,22 +660,16 @@ T *stage_out(Staging &s, T *host, size_t count) {
 // the arrays are gathered into (scattered from) a pinned buffer of the context,
 // laid out like the device staging area.  A copy of its own costs some 3 us on
 // the way to the copy engine and back, more than the CPU needs for 100 KB.
-// Two buffers take turns, so that a call can gather its inputs while the
-// copy of the call before it is still under way; larger calls copy every array
-// directly.  317 particles in and out of a step on 16384: 120 -> 74 us.
+// Larger calls copy every array directly.
 constexpr size_t kPackedStageBytes = 256 * 1024;
 
-// The next pinned buffer, free for writing; null if there is none (too large, or no memory).
+// The pinned buffer, free for writing; null if there is none (too large, or no memory).
 unsigned char *host_stage(sp2_ctx *c, size_t bytes) {
     if (bytes > 2 * kPackedStageBytes) return nullptr;
-    HostStage &h = c->hstage[c->hstage_next ^= 1];
-    if (!h.ev && cudaEventCreateWithFlags(&h.ev, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        h.ev = nullptr;
-        return nullptr;
-    }
-    if (h.pending && cudaEventSynchronize(h.ev) != cudaSuccess) return nullptr;
-    h.pending = false;
+    HostStage &h = c->hstage;
+    // (every call waits for its copies before it returns, unless it failed half-way)
+    if (h.busy && cudaStreamSynchronize(c->stream) != cudaSuccess) return nullptr;
+    h.busy = false;
     if (bytes > h.cap) {
         if (h.buf) cudaFreeHost(h.buf);
         h.cap = 0;
@@ -714,22 +706,22 @@ sp2_status stage_copy_in(Staging &s) {
         s.packed = true;
         for (size_t k = 0; k < s.in.size(); ++k)
             std::memcpy(s.host + (static_cast<unsigned char *>(s.in[k].first) - s.c->stage), s.in[k].second, s.in_bytes[k]);
+        s.c->hstage.busy = true;
         SP2_CK(s.c, cudaMemcpyAsync(s.c->stage + lo, s.host + lo, hi - lo, cudaMemcpyHostToDevice, s.c->stream));
-        HostStage &h = s.c->hstage[s.c->hstage_next];
-        SP2_CK(s.c, cudaEventRecord(h.ev, s.c->stream));
-        h.pending = true;
         return SP2_OK;
     }
     for (size_t k = 0; k < s.in.size(); ++k)
         SP2_CK(s.c, cudaMemcpyAsync(s.in[k].first, s.in[k].second, s.in_bytes[k], cudaMemcpyHostToDevice, s.c->stream));
     return SP2_OK;
 }
+// The call's outputs, if any, and the end of a host-pointer call: the stream is idle.
 sp2_status stage_copy_out(Staging &s) {
     size_t lo, hi;
     stage_extent(s, s.out, s.out_bytes, [](const std::pair<void *, void *> &q) { return q.second; }, lo, hi);
     if (s.packed && !s.out.empty() && hi - lo <= kPackedStageBytes) {
         SP2_CK(s.c, cudaMemcpyAsync(s.host + lo, s.c->stage + lo, hi - lo, cudaMemcpyDeviceToHost, s.c->stream));
         SP2_CK(s.c, cudaStreamSynchronize(s.c->stream));
+        s.c->hstage.busy = false;
         for (size_t k = 0; k < s.out.size(); ++k)
             std::memcpy(s.out[k].first, s.host + (static_cast<unsigned char *>(s.out[k].second) - s.c->stage), s.out_bytes[k]);
         return SP2_OK;
@@ -737,6 +729,7 @@ sp2_status stage_copy_out(Staging &s) {
     for (size_t k = 0; k < s.out.size(); ++k)
         SP2_CK(s.c, cudaMemcpyAsync(s.out[k].first, s.out[k].second, s.out_bytes[k], cudaMemcpyDeviceToHost, s.c->stream));
     SP2_CK(s.c, cudaStreamSynchronize(s.c->stream));
+    s.c->hstage.busy = false;
     return SP2_OK;
 }
 
@@ -912,10 +905,7 @@ sp2_status sp2_close(sp2_ctx *c) {
     for (cudaEvent_t e : c->blk_ev)
         if (e) cudaEventDestroy(e);
     if (c->blk_host) cudaFreeHost(c->blk_host);
-    for (HostStage &h : c->hstage) {
-        if (h.ev) cudaEventDestroy(h.ev);
-        if (h.buf) cudaFreeHost(h.buf);
-    }
+    if (c->hstage.buf) cudaFreeHost(c->hstage.buf);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
     return SP2_OK;
@@ -990,8 +980,7 @@ sp2_status sp2_set_j(sp2_ctx *c, int64_t first, int64_t n, const int32_t *slots,
             SP2_CK(c, launch_scatter_j(c->js, dsl, n, c->n_loaded, c->dev_words + 1, did, dm, dx, dv, da, dj, ds, dt, c->stream));
             ev_end(c, ST_OTHER);
             c->launches += 1;
-            // packed inputs have left the caller's arrays already
-            if (!s.packed) SP2_CK(c, cudaStreamSynchronize(c->stream));
+            SP2_CKS(stage_copy_out(s));  // (no outputs: waits for the scatter)
         }
     } else {
         if (!slots) {
