@@ -74,7 +74,8 @@ struct sp2_ctx {
     int32_t *iota = nullptr;
     double *tmp = nullptr;          // 4 x (n_max x 3) doubles: a1, j1, xpbar, vpbar
     unsigned int *dev_words = nullptr;  // [1] error flag, [2] finite flag; self-resetting: [0] batched work queue,
-                                        // [6] batched exit count, [4] pass work queue, [5] pass exit count
+                                        // [6] batched exit count, [4] pass work queue, [5] pass exit count;
+                                        // [8] no contents: cleared for the sake of the operation (stage_copy_in)
     double *part = nullptr;
     int32_t *part_id = nullptr;
     size_t part_cap = 0, part_id_cap = 0;   // bytes
@@ -628,8 +629,7 @@ struct Staging {
     std::vector<std::pair<void *, void *>> out;          // (host, device)
     std::vector<size_t> out_bytes;
     size_t total = 0;
-    unsigned char *host = nullptr;  // pinned image of the staging area (packed calls)
-    bool packed = false;
+    unsigned char *host = nullptr;  // pinned image of the staging area, once it holds the inputs
     void plan(size_t bytes) { total += (bytes + 255) / 256 * 256; }
     template <class T>
     T *slot(size_t bytes) {
@@ -660,7 +660,12 @@ T *stage_out(Staging &s, T *host, size_t count) {
 // the arrays are gathered into (scattered from) a pinned buffer of the context,
 // laid out like the device staging area.  A copy of its own costs some 3 us on
 // the way to the copy engine and back, more than the CPU needs for 100 KB.
-// Larger calls copy every array directly.
+// Larger calls copy every array directly, and a single input needs no gathering.
+// A copy in the stream reads a pinned (or managed) array only when its turn
+// comes, which may be the target of a copy that the caller queued before; the CPU
+// would be too early.  For such inputs an operation of the stream is waited for first
+// (one of its own: the stream may be one that runs behind the default stream's
+// work).  Pageable arrays are read when the call is made either way.
 constexpr size_t kPackedStageBytes = 256 * 1024;
 
 // The pinned buffer, free for writing; null if there is none (too large, or no memory).
@@ -701,9 +706,15 @@ void stage_extent(const Staging &s, const Pairs &v, const std::vector<size_t> &b
 sp2_status stage_copy_in(Staging &s) {
     size_t lo, hi;
     stage_extent(s, s.in, s.in_bytes, [](const std::pair<void *, const void *> &q) { return q.first; }, lo, hi);
-    s.packed = false;
-    if (!s.in.empty() && hi - lo <= kPackedStageBytes && (s.host = host_stage(s.c, s.total)) != nullptr) {
-        s.packed = true;
+    const bool pack = s.in.size() > 1 && hi - lo <= kPackedStageBytes;
+    cudaPointerAttributes at{};  // of the first array that the runtime knows
+    for (size_t k = 0; pack && k < s.in.size() && at.type == cudaMemoryTypeUnregistered; ++k)
+        SP2_CK(s.c, cudaPointerGetAttributes(&at, s.in[k].second));
+    if (pack && at.type != cudaMemoryTypeDevice && (s.host = host_stage(s.c, s.total)) != nullptr) {
+        if (at.type != cudaMemoryTypeUnregistered) {
+            SP2_CK(s.c, cudaMemsetAsync(s.c->dev_words + 8, 0, sizeof(unsigned int), s.c->stream));
+            SP2_CK(s.c, cudaStreamSynchronize(s.c->stream));
+        }
         for (size_t k = 0; k < s.in.size(); ++k)
             std::memcpy(s.host + (static_cast<unsigned char *>(s.in[k].first) - s.c->stage), s.in[k].second, s.in_bytes[k]);
         s.c->hstage.busy = true;
@@ -718,7 +729,8 @@ sp2_status stage_copy_in(Staging &s) {
 sp2_status stage_copy_out(Staging &s) {
     size_t lo, hi;
     stage_extent(s, s.out, s.out_bytes, [](const std::pair<void *, void *> &q) { return q.second; }, lo, hi);
-    if (s.packed && !s.out.empty() && hi - lo <= kPackedStageBytes) {
+    if (!s.host && s.out.size() > 1 && hi - lo <= kPackedStageBytes) s.host = host_stage(s.c, s.total);
+    if (s.host && !s.out.empty() && hi - lo <= kPackedStageBytes) {
         SP2_CK(s.c, cudaMemcpyAsync(s.host + lo, s.c->stage + lo, hi - lo, cudaMemcpyDeviceToHost, s.c->stream));
         SP2_CK(s.c, cudaStreamSynchronize(s.c->stream));
         s.c->hstage.busy = false;
