@@ -337,7 +337,8 @@ sp2_status sp2_set_launch(sp2_ctx *ctx, int64_t n_i, const sp2_launch *in);
 /* CUDA-graph capture of a sequence of calls on the context's stream (device
  * pointers only inside the capture; host-pointer calls return SP2_ERR_STATE).
  * sp2_graph_launch replays the captured calls with the same pointers and
- * arguments. */
+ * arguments.  Other calls, larger ones too, may run between the replays: scratch
+ * that the graph uses stays allocated until every graph is destroyed. */
 sp2_status sp2_graph_begin(sp2_ctx *ctx);
 sp2_status sp2_graph_end(sp2_ctx *ctx, sp2_graph **graph);
 sp2_status sp2_graph_launch(sp2_ctx *ctx, const sp2_graph *graph);

@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -35,6 +36,7 @@ constexpr size_t kSmemPerSm = 228 * 1024;  // shared memory of an SM
 struct sp2_graph {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    std::shared_ptr<int> live;  // the context's count of graphs (which outlives the context here)
 };
 
 struct sp2_batch_plan {
@@ -97,6 +99,8 @@ struct sp2_ctx {
     size_t stage_cap = 0;
     HostStage hstage;                // its pinned image (host_stage)
     std::vector<void *> owned;       // everything allocated (for close)
+    std::shared_ptr<int> live_graphs = std::make_shared<int>(0);  // graphs of this context not yet destroyed
+    std::vector<void *> retired;     // buffers that grew while one of them might still use the old address
 
     std::map<int64_t, sp2_launch> tuned;  // key: tune_key(n_i, n_j)
     std::map<std::array<int64_t, 5>, sp2_launch> shapes;  // default shapes of the sizes seen (shape_for)
@@ -197,14 +201,25 @@ sp2_status materialize(sp2_ctx *c) {
     return SP2_OK;
 }
 
-// Grow-only device buffer; refused while a graph is being captured.
+// Frees the outgrown buffers once no graph is left that could use them (on an idle stream).
+void free_retired(sp2_ctx *c) {
+    if (*c->live_graphs > 0) return;
+    for (void *p : c->retired) dfree(c, p);
+    c->retired.clear();
+}
+
+// Grow-only device buffer; refused while a graph is being captured.  A captured
+// graph holds the addresses of its capture, so while graphs exist an outgrown buffer
+// stays allocated: each is at most two thirds of its successor, so all
+// of them together are less than twice the last.
 sp2_status ensure(sp2_ctx *c, void **buf, size_t *cap, size_t need, const char *what) {
     if (need <= *cap) return SP2_OK;
     if (c->capturing)
         return fail(c, SP2_ERR_STATE, "%s scratch (%zu bytes) must be sized by one call before graph capture", what, need);
     size_t n = std::max(need, *cap + *cap / 2);
     SP2_CK(c, cudaStreamSynchronize(c->stream));
-    dfree(c, *buf);
+    if (*buf) c->retired.push_back(*buf);
+    free_retired(c);
     *buf = nullptr;
     *cap = 0;
     void *p = dalloc(c, n);
@@ -1767,6 +1782,8 @@ sp2_status sp2_graph_end(sp2_ctx *c, sp2_graph **out) {
         delete g;
         return cuda_fail(c, e, "graph capture");
     }
+    g->live = c->live_graphs;
+    *g->live += 1;
     *out = g;
     return SP2_OK;
 }
@@ -1782,6 +1799,7 @@ sp2_status sp2_graph_destroy(sp2_graph *g) {
     if (!g) return SP2_OK;
     if (g->exec) cudaGraphExecDestroy(g->exec);
     if (g->graph) cudaGraphDestroy(g->graph);
+    *g->live -= 1;
     delete g;
     return SP2_OK;
 }
@@ -1792,6 +1810,7 @@ sp2_status sp2_sync(sp2_ctx *c) {
     unsigned int flag = 0;
     SP2_CK(c, cudaMemcpyAsync(&flag, c->dev_words + 1, sizeof flag, cudaMemcpyDeviceToHost, c->stream));
     SP2_CK(c, cudaStreamSynchronize(c->stream));
+    free_retired(c);
     if (flag) {
         SP2_CK(c, cudaMemsetAsync(c->dev_words + 1, 0, sizeof flag, c->stream));
         SP2_CK(c, cudaStreamSynchronize(c->stream));
