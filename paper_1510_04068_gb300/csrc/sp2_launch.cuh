@@ -38,7 +38,9 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, u
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here, and not once more by the next launch of some other context
+    return e;
 }
 
 }  // namespace sp2

@@ -743,15 +743,13 @@ cudaError_t launch_scatter_j(const JStore &dst, const int32_t *slots, int64_t n,
                              const int32_t *id, const double *m, const double *x, const double *v, const double *a,
                              const double *jk, const double *sn, const double *t, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    launch_overlapped(scatter_kernel, grid_for_store(n), kSmallThreads, 0, s, dst, slots, n, n_loaded, err, id, m, x, v, a, jk, sn, t);
-    return cudaGetLastError();
+    return launch_overlapped(scatter_kernel, grid_for_store(n), kSmallThreads, 0, s, dst, slots, n, n_loaded, err, id, m, x, v, a, jk, sn, t);
 }
 
 cudaError_t launch_dscache(int order, const JStore &js, int64_t first, int64_t n, cudaStream_t s) {
     if (n <= 0 || !js.dsc) return cudaSuccess;
     (void)order;
-    launch_overlapped(dscache_kernel, grid_for_store(n), kSmallThreads, 0, s, js, first, n);
-    return cudaGetLastError();
+    return launch_overlapped(dscache_kernel, grid_for_store(n), kSmallThreads, 0, s, js, first, n);
 }
 
 namespace {
@@ -762,24 +760,22 @@ cudaError_t launch_predict_form(int order, int mixed, const JStore &js, int64_t 
     if (mixed && js.dsc) {
         const float th = static_cast<float>(t);
         const float tl = static_cast<float>(t - static_cast<double>(th));
-        if (order == 6) launch_overlapped(predict_ds_kernel<6, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
-        else if (order == 2) launch_overlapped(predict_ds_kernel<2, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
-        else launch_overlapped(predict_ds_kernel<4, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
-        return cudaGetLastError();
+        if (order == 6) return launch_overlapped(predict_ds_kernel<6, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
+        else if (order == 2) return launch_overlapped(predict_ds_kernel<2, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
+        return launch_overlapped(predict_ds_kernel<4, BLOCK>, g, kThreads, 0, s, js.dsc, n, th, tl, rec, b);
     }
     // the FP64 predictor is FP64-bound: 64-thread CTAs spread it over the SMs
     const unsigned g64 = static_cast<unsigned>((n + 63) / 64);
     if (order == 6) {
-        if (mixed) launch_overlapped(predict_kernel<6, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
-        else launch_overlapped(predict_kernel<6, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        if (mixed) return launch_overlapped(predict_kernel<6, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        return launch_overlapped(predict_kernel<6, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
     } else if (order == 2) {
-        if (mixed) launch_overlapped(predict_kernel<2, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
-        else launch_overlapped(predict_kernel<2, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        if (mixed) return launch_overlapped(predict_kernel<2, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        return launch_overlapped(predict_kernel<2, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
     } else {
-        if (mixed) launch_overlapped(predict_kernel<4, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
-        else launch_overlapped(predict_kernel<4, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        if (mixed) return launch_overlapped(predict_kernel<4, true, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
+        return launch_overlapped(predict_kernel<4, false, BLOCK>, g64, 64, 0, s, js, n, t, rec, b);
     }
-    return cudaGetLastError();
 }
 }  // namespace
 
@@ -798,9 +794,8 @@ cudaError_t launch_block_predict(int order, int mixed, const JStore &js, int64_t
 cudaError_t launch_pack_state(int mixed, int64_t n, const double *m, const double *x, const double *v,
                               unsigned char *rec, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (mixed) launch_overlapped(pack_state_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, rec);
-    else launch_overlapped(pack_state_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, rec);
-    return cudaGetLastError();
+    if (mixed) return launch_overlapped(pack_state_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, rec);
+    return launch_overlapped(pack_state_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, rec);
 }
 
 cudaError_t launch_pack_sinks(int order, int mixed, int64_t n, const double *x, const double *v, const double *a,
@@ -834,8 +829,7 @@ cudaError_t launch_block_correct_dev(const JStore &js, const BlockStep &b, int64
     if (n_max <= 0) return cudaSuccess;
     // (most blocks hold a small part of the particles: the grid is capped, and strides)
     const unsigned g = std::min(grid_for_warps(kLanesPerParticle * n_max), kCorrectMaxCtas);
-    launch_overlapped(block_correct_dev_kernel, g, kWarpCta, 0, s, js, b, a1, j1, eta, dt_max);
-    return cudaGetLastError();
+    return launch_overlapped(block_correct_dev_kernel, g, kWarpCta, 0, s, js, b, a1, j1, eta, dt_max);
 }
 
 cudaError_t launch_block_correct6_dev(const JStore &js, const BlockStep &b, int64_t n_max, const double *a1,
@@ -856,49 +850,43 @@ cudaError_t launch_block_init(const JStore &js, double *dt, int64_t n, double et
 cudaError_t launch_nb_finish(const int32_t *ids, int64_t n_i, int nb_max, const int32_t *count, int32_t *list,
                              cudaStream_t s) {
     if (n_i <= 0) return cudaSuccess;
-    launch_overlapped(nb_finish_kernel, static_cast<unsigned>((n_i + kNbWarps - 1) / kNbWarps), 32 * kNbWarps, 0, s, ids, n_i, nb_max, count, list);
-    return cudaGetLastError();
+    return launch_overlapped(nb_finish_kernel, static_cast<unsigned>((n_i + kNbWarps - 1) / kNbWarps), 32 * kNbWarps, 0, s, ids, n_i, nb_max, count, list);
 }
 
 cudaError_t launch_h4_predict_pack(int mixed, int64_t n, double dt, const double *m, const double *x,
                                    const double *v, const double *a, const double *jk, unsigned char *rec,
                                    cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (mixed) launch_overlapped(h4_predict_pack_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, rec);
-    else launch_overlapped(h4_predict_pack_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, rec);
-    return cudaGetLastError();
+    if (mixed) return launch_overlapped(h4_predict_pack_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, rec);
+    return launch_overlapped(h4_predict_pack_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, rec);
 }
 
 cudaError_t launch_h4_correct(int64_t n, double dt, double *x, double *v, double *a, double *jk, const double *a1,
                               const double *j1, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    launch_overlapped(h4_correct_kernel, grid_small(3 * n), kSmallThreads, 0, s, 3 * n, dt, x, v, a, jk, a1, j1);
-    return cudaGetLastError();
+    return launch_overlapped(h4_correct_kernel, grid_small(3 * n), kSmallThreads, 0, s, 3 * n, dt, x, v, a, jk, a1, j1);
 }
 
 cudaError_t launch_h4_vjp_pre(int mixed, int64_t n, double dt, const double *m, const double *x, const double *v,
                               const double *a, const double *jk, const double *gx, const double *gv,
                               const double *ga, const double *gj, unsigned char *vrec, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (mixed) launch_overlapped(h4_vjp_pre_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, gx, gv, ga, gj, vrec);
-    else launch_overlapped(h4_vjp_pre_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, gx, gv, ga, gj, vrec);
-    return cudaGetLastError();
+    if (mixed) return launch_overlapped(h4_vjp_pre_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, gx, gv, ga, gj, vrec);
+    return launch_overlapped(h4_vjp_pre_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, dt, m, x, v, a, jk, gx, gv, ga, gj, vrec);
 }
 
 cudaError_t launch_h4_vjp_post(int64_t n, double dt, const double *xpbar, const double *vpbar, double *gx,
                                double *gv, double *ga, double *gj, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    launch_overlapped(h4_vjp_post_kernel, grid_small(3 * n), kSmallThreads, 0, s, 3 * n, dt, xpbar, vpbar, gx, gv, ga, gj);
-    return cudaGetLastError();
+    return launch_overlapped(h4_vjp_post_kernel, grid_small(3 * n), kSmallThreads, 0, s, 3 * n, dt, xpbar, vpbar, gx, gv, ga, gj);
 }
 
 cudaError_t launch_pack_vjp(int mixed, int64_t n, const double *m, const double *x, const double *v,
                             const double *abar, const double *jbar, const double *pbar, unsigned char *vrec,
                             cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (mixed) launch_overlapped(pack_vjp_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, abar, jbar, pbar, vrec);
-    else launch_overlapped(pack_vjp_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, abar, jbar, pbar, vrec);
-    return cudaGetLastError();
+    if (mixed) return launch_overlapped(pack_vjp_kernel<true>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, abar, jbar, pbar, vrec);
+    return launch_overlapped(pack_vjp_kernel<false>, grid_small(n), kSmallThreads, 0, s, n, m, x, v, abar, jbar, pbar, vrec);
 }
 
 cudaError_t launch_scan_finite(const double *p, int64_t n, unsigned int *flag, cudaStream_t s) {
