@@ -81,6 +81,7 @@ struct sp2_ctx {
     double *part = nullptr;
     int32_t *part_id = nullptr;
     size_t part_cap = 0, part_id_cap = 0;   // bytes
+    size_t part_refused = ~size_t(0);       // smallest need of partial sums that could not be allocated
     unsigned int *done = nullptr;           // per-i-block arrival counters of the fused reduction
     size_t done_cap = 0;                    // bytes
     unsigned char *sinkrec = nullptr;       // records of explicit sinks
@@ -445,14 +446,12 @@ sp2_launch shape_for(sp2_ctx *c, int kind, int order, int mixed, int64_t n_i, in
 // fit one i-block predicts its sources from the double-single cache inside the
 // pass (each source is predicted once); otherwise deferred records are written
 // first.
-sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const unsigned char *rec, int rb,
-                    int64_t n_valid, const int32_t *i_idx, int64_t n_i, int64_t j_begin, int64_t j_end,
-                    const PassOut &o, const sp2_launch *forced, int stage_force, float *ms_out = nullptr,
-                    bool allow_fused = false, const unsigned int *n_i_dev = nullptr) {
-    if (n_i <= 0) return SP2_OK;
-    const int nb = (kind == K_FORCE && nn && o.nb_count) ? 1 : 0;
-    int64_t group = 0;  // group of the mixed sums that slices may not cut (0: none)
-    sp2_launch L = forced ? *forced : shape_for(c, kind, order, mixed, n_i, j_end - j_begin, nn, nb, &group);
+// group: sources of a group of the mixed sums, which slices may not cut (0: none);
+// part_limit: bytes of partial sums from which on the call fails (SP2_ERR_NOMEM).
+sp2_status run_shaped_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const unsigned char *rec, int rb,
+                           int64_t n_valid, const int32_t *i_idx, int64_t n_i, int64_t j_begin, int64_t j_end,
+                           const PassOut &o, sp2_launch L, int64_t group, size_t part_limit, int nb, int stage_force,
+                           float *ms_out, bool allow_fused, const unsigned int *n_i_dev) {
     if (nb) L.i_per_thread = 1;  // neighbour-list kernels take one sink per thread
     const int64_t n_j = j_end - j_begin;
     const int jl = L.j_lanes;
@@ -579,9 +578,13 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
     const int ns = ns_fields;
     if (split > 1) {
         const size_t need = static_cast<size_t>(ns + (nn ? 1 : 0)) * split * n_part * sizeof(double);
-        SP2_CKS(ensure(c, reinterpret_cast<void **>(&c->part), &c->part_cap, need, "partial-sum"));
-        if (nn) SP2_CKS(ensure(c, reinterpret_cast<void **>(&c->part_id), &c->part_id_cap,
-                               static_cast<size_t>(split) * n_part * sizeof(int32_t), "partial-id"));
+        if (need >= part_limit) return fail(c, SP2_ERR_NOMEM, "%zu bytes of partial-sum scratch were refused before", need);
+        sp2_status st = ensure(c, reinterpret_cast<void **>(&c->part), &c->part_cap, need, "partial-sum");
+        if (st == SP2_OK && nn)
+            st = ensure(c, reinterpret_cast<void **>(&c->part_id), &c->part_id_cap,
+                        static_cast<size_t>(split) * n_part * sizeof(int32_t), "partial-id");
+        if (st == SP2_ERR_NOMEM) c->part_refused = std::min(c->part_refused, need);
+        SP2_CKS(st);
         p.part = c->part;
         p.part_id = c->part_id;
         // A device-count pass reduces its slices itself (no host knows how many
@@ -633,6 +636,27 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
         *ms_out = ms;
     }
     return SP2_OK;
+}
+
+// The same with a given shape or the one for these sizes.  The default shapes take
+// as many slices as serve the speed (up to some 200 MB of partial sums); where
+// the memory for that is refused, fewer slices do the same work more slowly (the
+// context does not ask for as much again).
+sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const unsigned char *rec, int rb,
+                    int64_t n_valid, const int32_t *i_idx, int64_t n_i, int64_t j_begin, int64_t j_end,
+                    const PassOut &o, const sp2_launch *forced, int stage_force, float *ms_out = nullptr,
+                    bool allow_fused = false, const unsigned int *n_i_dev = nullptr) {
+    if (n_i <= 0) return SP2_OK;
+    const int nb = (kind == K_FORCE && nn && o.nb_count) ? 1 : 0;
+    int64_t group = 0;
+    sp2_launch L = forced ? *forced : shape_for(c, kind, order, mixed, n_i, j_end - j_begin, nn, nb, &group);
+    const bool given = forced || (kind == K_FORCE && c->tuned.count(tune_key(n_i, j_end - j_begin)));
+    for (;; L.split_j /= 2) {
+        const sp2_status st = run_shaped_pass(c, kind, order, mixed, nn, rec, rb, n_valid, i_idx, n_i, j_begin, j_end, o,
+                                              L, group, given ? ~size_t(0) : c->part_refused, nb, stage_force, ms_out,
+                                              allow_fused, n_i_dev);
+        if (st != SP2_ERR_NOMEM || given || L.split_j <= 1) return st;
+    }
 }
 
 // Host-pointer staging helpers.
