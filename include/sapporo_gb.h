@@ -28,11 +28,11 @@
  *    and the pair with itself is skipped.  Particle ids must be unique; the
  *    nearest-neighbour output reports the neighbour's id.
  *  - Precision: SP2_FP64 computes everything in IEEE double.  SP2_MIXED
- *    predicts in FP64, stores positions as double-single (FP32 hi + lo) pairs,
- *    forms x_j - x_i in double-single, evaluates rsqrt and the force terms in
- *    FP32, and accumulates per-thread partial sums in FP32 that are flushed
- *    into FP64 every tile; partial results of different j-slices are combined
- *    in FP64.
+ *    predicts in double-single (FP32 hi + lo pairs), forms x_j - x_i in
+ *    double-single, evaluates rsqrt and the force terms in FP32, and
+ *    accumulates per-thread partial sums in FP32 that go into double-single
+ *    totals every 64 sources or more; partial results of different j-slices
+ *    are combined in FP64.
  */
 #ifndef SAPPORO_GB_H
 #define SAPPORO_GB_H
@@ -152,8 +152,10 @@ sp2_status sp2_predict(sp2_ctx *ctx, double t);
  * Any output may be NULL (not computed / not written); nn_* need with_nn.
  * Sinks are the predicted j-particles at t.  The source range is split into
  * slices over the whole GPU when n_i is small (Sec. 2.1, the source-split
- * method), and the slices are combined by a deterministic FP64 reduction
- * (inside the force kernel, or a second kernel for large slice counts).
+ * method), and the slices are combined by a deterministic FP64 reduction (a
+ * second kernel).  The partial sums take up to some 200 MB of scratch, allocated by
+ * the first call that needs as much; where that is refused, the default launch
+ * shape takes fewer slices.
  * Errors: SP2_ERR_STATE (records stale: call sp2_predict),
  * SP2_ERR_RANGE (slot >= loaded count, bad range), SP2_ERR_ARG,
  * SP2_ERR_NONFINITE (check_finite). n_i == 0 is a successful no-op. */

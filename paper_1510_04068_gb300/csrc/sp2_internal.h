@@ -126,14 +126,20 @@ constexpr int kMaxPassSmem = 222 * 1024;
 // adjoint) or in one word's four (order 6: eight-way conflicts); one word of
 // padding makes the stride odd, and they cover all banks once.  With fewer lanes
 // the distinct words of a load do not conflict, and the larger tile would only
-// cost resident CTAs (measured: 13 % at 16384 sinks with two lanes each).
-// 61 sinks on 131072 sources (8 lanes each) 49 -> 45 us a step; a block run of
-// 4096 particles (32 lanes) 1.62 -> 1.75 times the speed of its first form.
+// cost resident CTAs (measured: 13 % at 16384 sinks with two lanes each).  The kernels
+// with two sinks per thread go without (a stride that is not a constant
+// cost the full-size pass a register).  A step without / with it: 20 sinks on
+// 131072 sources (16 lanes) 28.7 / 24.7 us, 8 sinks (32 lanes) 14.5 / 13.1 us, 8 sinks on
+// 65536 at order 6 21.6 / 13.7 us; an order-6 block run of 4096 particles 1.73 / 1.54 ms
+// (order 4: the same).
 constexpr int kPairPad = 16;
 constexpr int kPairPadMinLanes = 8;
 
 // From this many slices on, the split-j reduction divides a column's slices
-// over several threads.
+// over several threads.  One thread / several per column, us a step: 8 sinks on 16384
+// sources (32 slices) 13.4 / 10.9, 317 sinks (64) 29.3 / 24.0, 1000 on 100003
+// (112) 180 / 168; below, 12000 sinks on 16384 (19 slices) 307 / 320, 1024 on 1024
+// in FP64 (16) 82.0 / 83.1.
 constexpr int kGroupReduceMinSplit = 32;
 
 struct KernelKey {

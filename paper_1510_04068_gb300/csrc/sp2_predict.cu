@@ -32,6 +32,8 @@ inline unsigned grid_for(int64_t n) { return static_cast<unsigned>((n + kThreads
 // FP64-heavy per-particle kernels over a few hundred active particles: one
 // warp per CTA spreads them over the SMs (an SM retires 2 FP64 FMAs a clock)
 constexpr int kWarpCta = 32;
+// (256, 2048 or as many CTAs as the particles need: block runs of 4096 and 65536
+// particles differ by less than two runs of one of them)
 constexpr unsigned kCorrectMaxCtas = 2048;
 inline unsigned grid_for_warps(int64_t n) { return static_cast<unsigned>((n + kWarpCta - 1) / kWarpCta); }
 
