@@ -48,11 +48,13 @@ struct sp2_batch_plan {
     int64_t max_size = 0;
 };
 
-// The pinned buffer of the host-pointer calls; busy: a copy out of it may be under way.
+// The pinned buffer of the host-pointer calls; busy: a copy out of it may be under
+// way; ev: waited for before pinned inputs are read.
 struct HostStage {
     unsigned char *buf = nullptr;
     size_t cap = 0;
     bool busy = false;
+    cudaEvent_t ev = nullptr;
 };
 
 struct sp2_ctx {
@@ -76,8 +78,7 @@ struct sp2_ctx {
     int32_t *iota = nullptr;
     double *tmp = nullptr;          // 4 x (n_max x 3) doubles: a1, j1, xpbar, vpbar
     unsigned int *dev_words = nullptr;  // [1] error flag, [2] finite flag; self-resetting: [0] batched work queue,
-                                        // [6] batched exit count, [4] pass work queue, [5] pass exit count;
-                                        // [8] no contents: cleared for the sake of the operation (stage_copy_in)
+                                        // [6] batched exit count, [4] pass work queue, [5] pass exit count
     double *part = nullptr;
     int32_t *part_id = nullptr;
     size_t part_cap = 0, part_id_cap = 0;   // bytes
@@ -420,13 +421,17 @@ int pair_pad_for(int kind, int order, int mixed, int tile, int rb, int threads, 
 
 // The shape of a pass: the tuned one for the bucket of its sizes, else the
 // default (a bounded table of those computed, keyed by sizes only; *group: see
-// grouping()).
+// grouping(); *tuned: it is the tuned one).
 sp2_launch shape_for(sp2_ctx *c, int kind, int order, int mixed, int64_t n_i, int64_t n_j, int nn, int nb,
-                     int64_t *group) {
+                     int64_t *group, bool *tuned) {
     *group = 0;
-    if (kind == K_FORCE) {
+    *tuned = false;
+    if (kind == K_FORCE && !c->tuned.empty()) {
         auto it = c->tuned.find(tune_key(n_i, n_j));
-        if (it != c->tuned.end()) return it->second;
+        if (it != c->tuned.end()) {
+            *tuned = true;
+            return it->second;
+        }
     }
     const Grouping g = grouping(c, kind, n_i, n_j);
     if (mixed) *group = g.group;
@@ -650,8 +655,8 @@ sp2_status run_pass(sp2_ctx *c, int kind, int order, int mixed, int nn, const un
     if (n_i <= 0) return SP2_OK;
     const int nb = (kind == K_FORCE && nn && o.nb_count) ? 1 : 0;
     int64_t group = 0;
-    sp2_launch L = forced ? *forced : shape_for(c, kind, order, mixed, n_i, j_end - j_begin, nn, nb, &group);
-    const bool given = forced || (kind == K_FORCE && c->tuned.count(tune_key(n_i, j_end - j_begin)));
+    bool given = true;
+    sp2_launch L = forced ? *forced : shape_for(c, kind, order, mixed, n_i, j_end - j_begin, nn, nb, &group, &given);
     for (;; L.split_j /= 2) {
         const sp2_status st = run_shaped_pass(c, kind, order, mixed, nn, rec, rb, n_valid, i_idx, n_i, j_begin, j_end, o,
                                               L, group, given ? ~size_t(0) : c->part_refused, nb, stage_force, ms_out,
@@ -702,13 +707,14 @@ T *stage_out(Staging &s, T *host, size_t count) {
 // the way to the copy engine and back, more than the CPU needs for 100 KB.
 // Larger calls copy every array directly, and a single input needs no gathering.
 // A step on 16384 sources from pinned arrays, a copy per array / packed: 17 particles
-// 81 / 67 us, 317 99 / 83, 900 117 / 111, 1900 (236 KB) 151 / 153, 4000 212 / 233; from
-// pageable arrays 317 particles 122 / 77, 1900 186 / 145.
+// 81 / 60 us, 317 100 / 78, 900 119 / 101, 1900 (236 KB) 154 / 148, 4000 214 / 225; from
+// pageable arrays 317 124 / 77, 1900 188 / 147, 4000 280 / 222, 12000 497 / 503.
 // A copy in the stream reads a pinned (or managed) array only when its turn
 // comes, which may be the target of a copy that the caller queued before; the CPU
-// would be too early.  For such inputs an operation of the stream is waited for first
-// (one of its own: the stream may be one that runs behind the default stream's
-// work).  Pageable arrays are read when the call is made either way.
+// would be too early.  For such inputs an event in the stream is waited for first
+// (synchronising the stream would not do: an idle blocking stream falls in behind
+// the default stream's work only with its next operation).  Pageable arrays are read
+// when the call is made either way.
 constexpr size_t kPackedStageBytes = 256 * 1024;
 
 // The pinned buffer, free for writing; null if there is none (too large, or no memory).
@@ -755,8 +761,10 @@ sp2_status stage_copy_in(Staging &s) {
         SP2_CK(s.c, cudaPointerGetAttributes(&at, s.in[k].second));
     if (pack && at.type != cudaMemoryTypeDevice && (s.host = host_stage(s.c, s.total)) != nullptr) {
         if (at.type != cudaMemoryTypeUnregistered) {
-            SP2_CK(s.c, cudaMemsetAsync(s.c->dev_words + 8, 0, sizeof(unsigned int), s.c->stream));
-            SP2_CK(s.c, cudaStreamSynchronize(s.c->stream));
+            cudaEvent_t &ev = s.c->hstage.ev;
+            if (!ev) SP2_CK(s.c, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+            SP2_CK(s.c, cudaEventRecord(ev, s.c->stream));
+            SP2_CK(s.c, cudaEventSynchronize(ev));
         }
         for (size_t k = 0; k < s.in.size(); ++k)
             std::memcpy(s.host + (static_cast<unsigned char *>(s.in[k].first) - s.c->stage), s.in[k].second, s.in_bytes[k]);
@@ -961,6 +969,7 @@ sp2_status sp2_close(sp2_ctx *c) {
         if (e) cudaEventDestroy(e);
     if (c->blk_host) cudaFreeHost(c->blk_host);
     if (c->hstage.buf) cudaFreeHost(c->hstage.buf);
+    if (c->hstage.ev) cudaEventDestroy(c->hstage.ev);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
     return SP2_OK;
@@ -1648,8 +1657,9 @@ sp2_status sp2_get_launch(sp2_ctx *c, int64_t n_i, sp2_launch *out) {
     SP2_CKS(usable(c));
     if (!out || n_i <= 0) return fail(c, SP2_ERR_ARG, "bad arguments");
     int64_t group;
+    bool tuned;
     *out = shape_for(c, K_FORCE, c->cfg.order, c->cfg.precision == SP2_MIXED, n_i, std::max<int64_t>(c->n_loaded, 1),
-                     c->cfg.with_nn, 0, &group);
+                     c->cfg.with_nn, 0, &group, &tuned);
     return SP2_OK;
 }
 
