@@ -2140,9 +2140,9 @@ __global__ void __launch_bounds__(kMaxThreads, (pass_min_blocks<P, IPT, FUSED>::
 // fewer slices take a thread per column.  The kernel is bound by the latency of
 // those trips.  Before, one warp per sink (or one thread) added the slices with
 // two loads in flight, inside the pass's last CTA up to 16384 partial sums:
-// 61 sinks on 131072 sources in 512 slices took 121 us for the step, now
-// 61 us; 317 on 16384 in 64 slices 222 us, now 121 us; the 16384-particle
-// adjoint run (32 slices) 18.4 ms, now 14.8 ms.
+// 61 sinks on 131072 sources in 512 slices took 121 us for the step, with this
+// form 61 us; 317 on 16384 in 64 slices 222 and 121 us; the 16384-particle
+// adjoint run (32 slices) 18.4 and 14.8 ms (default shapes of that time).
 // The line between 8 and 32 threads per column, us a step with 8 / with 32 on
 // either side of it: 1 sink on 131072 sources 14.1 / 12.4, 8 sinks 17.0 / 13.1, 61
 // sinks (488 columns) 37.1 / 35.1; 1000 sinks (8000 columns) 167 / 173, 4096 sinks
